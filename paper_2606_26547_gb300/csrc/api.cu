@@ -368,13 +368,9 @@ hdc_status hdc_hamming_argmin_ws(const uint32_t *Q, const uint32_t *Cls, int64_t
     if (!need)
         return cu(launch_similarity(Q, N, Cls, C, W, 1, D, perforated ? &p : nullptr, nullptr, nullptr, labels, dists,
                                     nullptr, st));
-    // the classes once into ws (zero past D; the query bytes are zero
-    // outside the kept dims), then the tensor-core route streams them
-    uint8_t *signs = (uint8_t *)ws;
-    hdc_status s = cu(launch_class_sign(Cls, C, W, D, (C + 15) / 16 * 16, hamming_packed_ldcs(W), signs, st));
-    if (s != HDC_OK) return s;
+    // the classes once into ws, then the tensor-core route streams them
     return cu(launch_hamming_packed(Q, N, Cls, C, W, D, perforated ? p.s0 : 0, perforated ? p.e0 : D,
-                                    perforated ? p.stride : 1, labels, dists, st, signs));
+                                    perforated ? p.stride : 1, labels, dists, st, (uint8_t *)ws));
 }
 
 namespace {
@@ -550,11 +546,8 @@ hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m, int32_t *
         if (s != HDC_OK) return s;
     }
     if (classify_sign_bytes(m)) {   // 129..256 binary classes: the classes expanded once, then the tensor cores
-        uint8_t *signs = (uint8_t *)ws + L.csign;
-        s = cu(launch_class_sign(m->cls, m->C, m->W, m->Dk, (m->C + 15) / 16 * 16, hamming_packed_ldcs(m->W), signs,
-                                 st));
-        if (s != HDC_OK) return s;
-        return cu(launch_hamming_packed(Hb, N, m->cls, m->C, m->W, m->Dk, 0, m->Dk, 1, labels, dists, st, signs));
+        return cu(launch_hamming_packed(Hb, N, m->cls, m->C, m->W, m->Dk, 0, m->Dk, 1, labels, dists, st,
+                                        (uint8_t *)ws + L.csign));
     }
     return cu(launch_similarity(Hb, N, m->cls, m->C, m->W, nb, m->Dk, nullptr, m->cls_sum, m->cls_norm, labels,
                                 dists, scores, st));

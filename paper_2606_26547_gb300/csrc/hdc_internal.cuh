@@ -192,16 +192,16 @@ cudaError_t quant_read_status(cudaStream_t st, int *status);
 
 // Reads and clears the tensor-core kernels' device status word.
 cudaError_t tc_read_status(cudaStream_t st, int *status);
-// Hamming arg-min of packed rows on the tensor cores (17 <= C <= 256 binary
+// Hamming arg-min of packed rows on the tensor cores (up to 256 binary
 // classes, W a multiple of 4 up to 4096): kept dims s0 + k*stride < min(e0, D).
 bool hamming_packed_ok(int C, int W);
-// cls_sign (optional): the class hypervectors already expanded by
-// launch_class_sign(cls, C, W, Dk, Cp, hamming_packed_ldcs(W), cls_sign) --
-// the kernel then streams them instead of expanding the class words itself.
+// signs (optional): Cp rows (C rounded up to 16) of hamming_packed_ldcs(W)
+// bytes, into which the class hypervectors are expanded once per call; without
+// it the kernel expands the class words of every tile itself.
 int hamming_packed_ldcs(int W);
 cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *cls, int C, int W, int64_t D,
                                   int64_t s0, int64_t e0, int64_t stride, int32_t *labels, int32_t *dists,
-                                  cudaStream_t st, const uint8_t *cls_sign = nullptr);
+                                  cudaStream_t st, uint8_t *signs = nullptr);
 // One block waiting, bounded by limit_ns, on a barrier nothing arrives on
 // (the expiry is reported through tc_read_status).
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st);

@@ -1,7 +1,7 @@
 // Auxiliary tensor-core kernels in a translation unit of their own (with
 // its own device status word): the Hamming arg-min of packed hypervectors
 // and the failure-detection self-test.
-#include <string.h>
+
 
 #include "tc_hamming_packed.cuh"
 
@@ -10,6 +10,9 @@ namespace hdc {
 // Tensor map of E4M3 class bytes (Cp rows of ldcs bytes, boxes of 128 bytes x
 // Cp rows, 128-byte swizzle), defined with the other map builders.
 bool make_class_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int Cp);
+// Tensor map of packed rows (N rows of W words): boxes of 32 words x 128 rows,
+// 128-byte swizzle, zeros past W and N.
+bool make_packed_map(CUtensorMap *m, const uint32_t *Q, int W, int64_t N);
 namespace tc {
 
 // Failure-detection self-test: thread 0 waits, through the bounded-wait
@@ -32,71 +35,135 @@ __global__ void __launch_bounds__(32, 1) wait_selftest_kernel(unsigned long long
 
 bool hamming_packed_ok(int C, int W)
 {
-    return C > 16 && C <= tc::HP_CMAX && W > 0 && W <= tc::HP_MAX_W && W % 4 == 0;
+    return C > 0 && C <= tc::HP_CMAX && W > 0 && W <= tc::HP_MAX_W && W % 4 == 0;
 }
 
 int hamming_packed_ldcs(int W) { return (W + 7) / 8 * 256; }
 
+namespace {
+// Class words -> E4M3 bytes in the packed kernel's dim order, zero outside
+// the kept dims: a thread writes the four dims j, j + 8, j + 16, j + 24 of one
+// word, 32 bytes a word.
+__global__ void class_bytes_kernel(const uint32_t *__restrict__ cls, int C, int W, int ldw, int64_t D, int64_t s0,
+                                   int64_t e0, int64_t stride, uint32_t *__restrict__ out)
+{
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (int64_t)C * ldw) return;
+    const int c = (int)(i / ldw), x = (int)(i % ldw), w = x >> 3, j = x & 7;
+    uint32_t v = 0;
+    if (w < W)
+        v = tc::hp_signs(__ldg(cls + (int64_t)c * W + w), j) & tc::hp_mask(tc::hp_word_mask(w, D, s0, e0, stride), j);
+    out[i] = v;
+}
+
+int hp_sms()
+{
+    int dev = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
+                                                     cudaSuccess || sms <= 0)
+        sms = 152;
+    return sms;
+}
+
+// Units (MT x 128 rows), CTAs per unit and the wave-time estimate of one form:
+// waves x 256-dim tiles per CTA x the tile's time.  A split needs its clusters
+// resident together: an SM group holds at least 16 SMs, so at most
+// 8 * floor(16 / S) clusters of S CTAs at once.
+struct HpPlan {
+    int mt, S;
+    int64_t units, cost;
+};
+HpPlan hp_plan(int64_t N, int mt, int chunks, int sms, int tile_cost)
+{
+    HpPlan pl;
+    pl.mt = mt;
+    pl.units = (N + mt * tc::BM - 1) / (mt * tc::BM);
+    pl.S = 1;
+    for (int S = 2; S <= tc::HP_SMAX && S <= chunks; S++)
+        if (pl.units * S <= sms && pl.units <= 8 * (16 / S)) pl.S = S;
+    const int64_t waves = (pl.units * pl.S + sms - 1) / sms;
+    pl.cost = waves * ((chunks + pl.S - 1) / pl.S) * tile_cost;
+    return pl;
+}
+}  // namespace
+
+// Form of a call.  Two 128-row tiles a unit halve the class bytes streamed per
+// row (R x D bytes a unit); one tile a unit fills the chip with half the rows
+// and is the only form past 128 class rows (two D2 of 256 columns do not fit).
+// The estimate weighs a 256-dim tile of two at 5 and of one at 3.  Measured,
+// replays of one call with the workspace, the two-CTA form before (one tile a
+// unit, its class tile copied inside the expand -> MMA chain, bit-transposing
+// expansion) -> this one:
+//   10^5 x 16,384 dims: 100 classes 226.5 -> 194.2 us, 256 classes 393 -> 279
+//   10^6 x 1,024 dims:  100 classes 206.6 -> 153.2 us, 33 classes 168 -> 115
+// and without the workspace (classes expanded per tile) 365 -> 258 us at 10^5
+// x 16,384 x 100.
 cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *cls, int C, int W, int64_t D,
                                   int64_t s0, int64_t e0, int64_t stride, int32_t *labels, int32_t *dists,
-                                  cudaStream_t st, const uint8_t *cls_sign)
+                                  cudaStream_t st, uint8_t *signs)
 {
     if (N <= 0) return cudaSuccess;
-    if (!hamming_packed_ok(C, W) || stride < 1) return cudaErrorNotSupported;
-    CUtensorMap mc;
-    memset(&mc, 0, sizeof(mc));
-    if (cls_sign && !make_class_sign_map(&mc, cls_sign, hamming_packed_ldcs(W), (C + 15) / 16 * 16))
-        return cudaErrorInvalidValue;
+    if (!hamming_packed_ok(C, W) || stride < 1 || N > 0x7fffffffLL - 2 * tc::BM) return cudaErrorNotSupported;
+    const int ldcs = hamming_packed_ldcs(W), R = (C + 15) / 16 * 16;
+    CUtensorMap mq, mc;
+    if (!make_packed_map(&mq, Q, W, N)) return cudaErrorInvalidValue;
+    mc = mq;
+    if (signs) {   // the classes once into `signs`, zero outside the kept dims
+        const int64_t n = (int64_t)C * (ldcs / 4);
+        class_bytes_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(cls, C, W, ldcs / 4, D, s0, e0, stride,
+                                                                        reinterpret_cast<uint32_t *>(signs));
+        const cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        if (!make_class_sign_map(&mc, signs, ldcs, R)) return cudaErrorInvalidValue;
+    }
     tc::HPParams p;
-    p.Q = Q;
     p.cls = cls;
     p.N = N;
     p.W = W;
     p.C = C;
-    p.Cp = (C + 15) / 16 * 16;
+    p.R = R;
     p.nt = (W + 7) / 8;
     p.D = D;
     p.s0 = s0;
     p.e0 = e0;
     p.stride = stride;
+    const int64_t end = e0 < D ? e0 : D;
+    p.kept = end > s0 ? (int)((end - s0 + stride - 1) / stride) : 0;
     p.labels = labels;
     p.dists = dists;
-    int dev = 0, sms = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) !=
-                                                     cudaSuccess || sms <= 0)
-        sms = 152;
-    const int64_t tiles = (N + tc::BM - 1) / tc::BM;
-    // Up to 128 padded classes the query tile lives in tensor memory, two
-    // CTAs per SM (256 TMEM columns each, two class-tile buffers).  Above,
-    // two CTAs per SM with the query tile in shared memory where they fit
-    // (two class-tile buffers, else one), else one CTA with the query tile in
-    // tensor memory and all 512 columns: measured, the two-CTA forms win up
-    // to ~176 classes (10^5 x 16,384 dims, 144 classes: 0.339 vs 0.377 ms)
-    // and the one-CTA tensor-memory form above (256 classes: 0.397 vs 0.459
-    // ms with the one-CTA shared-memory form).  The one-CTA form asks for at
-    // least 120 KB of shared memory, so that no second CTA shares the SM and
-    // waits for its 512 columns.
-    auto fits2 = [](size_t bytes) { return 2 * (bytes + 1024) <= 228 * 1024; };
-    const size_t smem2 = tc::hp_smem_bytes(p.Cp, W, 2), smem1 = tc::hp_smem_bytes(p.Cp, W, 1);
-    const size_t smta = tc::hp_smem_bytes(p.Cp, W, 2, true);
-    const int form = p.Cp <= tc::HP_TA_CMAX ? 0 : fits2(smem2) ? 1 : fits2(smem1) ? 2 : 3;
-    const bool two = form < 3;
-    const size_t smem = form == 0 ? smta : form == 1 ? smem2 : form == 2 ? smem1
-                      : (smta >= (size_t)120 * 1024 ? smta : (size_t)120 * 1024);
-    auto k = cls_sign ? (form == 0   ? tc::tc_hamming_packed_kernel<2, 2, true, true>
-                         : form == 1 ? tc::tc_hamming_packed_kernel<2, 2, true>
-                         : form == 2 ? tc::tc_hamming_packed_kernel<2, 1, true>
-                                     : tc::tc_hamming_packed_kernel<1, 2, true, true>)
-                      : (form == 0   ? tc::tc_hamming_packed_kernel<2, 2, false, true>
-                         : form == 1 ? tc::tc_hamming_packed_kernel<2, 2, false>
-                         : form == 2 ? tc::tc_hamming_packed_kernel<2, 1, false>
-                                     : tc::tc_hamming_packed_kernel<1, 2, false, true>);
+    const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
+    HpPlan pl = hp_plan(N, 1, chunks, sms, 3);
+    if (R <= 128) {
+        const HpPlan p2 = hp_plan(N, 2, chunks, sms, 5);
+        if (p2.cost < pl.cost) pl = p2;
+    }
+    p.S = pl.S;
+    // shared memory: the query ring, the class atoms, barriers; at least 120 KB
+    // so that no second CTA shares the SM and waits for its TMEM columns
+    const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::HP_TAIL, atom = (size_t)R * 128;
+    size_t nbs = (227 * 1024 - fixed) / atom;
+    if (nbs > (size_t)tc::HP_NBS_MAX) nbs = tc::HP_NBS_MAX;
+    p.nbs = (int)nbs;
+    size_t smem = fixed + (signs ? nbs * atom : 4 * atom + (size_t)((W + 3) & ~3) * 4);
+    if (smem < 120 * 1024) smem = 120 * 1024;
+    auto k = pl.mt == 2 ? (signs ? tc::tc_hamming_packed_kernel<2, true> : tc::tc_hamming_packed_kernel<2, false>)
+                        : (signs ? tc::tc_hamming_packed_kernel<1, true> : tc::tc_hamming_packed_kernel<1, false>);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const int64_t slots = (int64_t)sms * (two ? 2 : 1);
-    const unsigned grid = (unsigned)(tiles < slots ? tiles : slots);
-    k<<<grid, tc::HP_THREADS, smem, st>>>(p, mc);
-    return cudaGetLastError();
+    const int64_t ctas = pl.units * pl.S;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(pl.S > 1 || ctas < sms ? ctas : sms));
+    lc.blockDim = dim3(tc::HP_THREADS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)pl.S;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = pl.S > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, k, p, mq, mc);
 }
 
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st)

@@ -531,9 +531,6 @@ cudaError_t launch_argmin_ws(const uint32_t *H, int64_t N, const uint32_t *cls, 
     if (N <= 0) return cudaSuccess;
     if (signs && class_sign_bytes(C, W) > 0) {
         // expand the classes once, then stream them to the tensor-core route
-        const int Cp = (C + 15) / 16 * 16;
-        cudaError_t e = launch_class_sign(cls, C, W, (int)D, Cp, hamming_packed_ldcs(W), signs, st);
-        if (e != cudaSuccess) return e;
         return launch_hamming_packed(H, N, cls, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      nullptr, st, signs);
     }
