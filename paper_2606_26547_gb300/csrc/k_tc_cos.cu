@@ -88,7 +88,7 @@ __global__ void __launch_bounds__(192, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == 4) {
-        if (lane == 0) {  // ---------------------------------- TMA producer
+        if (elect_one()) {  // ---------------------------------- TMA producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
             int stage = 0;
@@ -99,7 +99,7 @@ __global__ void __launch_bounds__(192, 1)
             bool ab = false;
             for (int64_t mt = blockIdx.x; mt < num_m_tiles && !ab; mt += gridDim.x)
                 for (int kb = 0; kb < p.num_kb; kb++) {
-                    if (!mbar_wait(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
+                    if (!mbar_wait_fast(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
                     mbar_expect_tx(full(stage), CA_BYTES + b_bytes);
                     tma_load_2d(su32(sA + stage * CA_BYTES), &tmA, kb * (BKB / 2), (int)(mt * BM), full(stage));
                     tma_load_2d(su32(sB + stage * CB_MAX), &tmB, kb * (BKB / 2), 0, full(stage));
@@ -116,7 +116,7 @@ __global__ void __launch_bounds__(192, 1)
             }
         }
     } else if (warp == 5) {
-        if (lane == 0) {  // ---------------------------------- MMA issuer
+        if (elect_one()) {  // ---------------------------------- MMA issuer
             // BF16 x BF16 -> FP32, K-major A and B, M = 128, N = Cp
             const uint32_t id = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(p.Cp >> 3) << 17) |
                                 ((uint32_t)(BM >> 4) << 24);

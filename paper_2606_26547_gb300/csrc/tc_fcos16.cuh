@@ -141,7 +141,7 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == PRODUCER) {
-        if (lane == 0) {  // ------------------------------ A / B stage producer
+        if (elect_one()) {  // ------------------------------ A / B stage producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
             int stage = 0;
@@ -153,7 +153,7 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
             for (int64_t mt = blockIdx.x; mt < num_m_tiles && !ab; mt += gridDim.x)
                 for (int t = 0; t < p.nt && !ab; t++)
                     for (int kb = 0; kb < p.num_kb; kb++) {
-                        if (!mbar_wait(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
+                        if (!mbar_wait_fast(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
                         mbar_expect_tx(full(stage), STAGE_BYTES);
                         tma_load_2d(su32(sA + stage * A_BYTES), &tmA, kb * KELEMS, (int)(mt * BM), full(stage));
                         tma_load_2d(su32(sB + stage * B_BYTES), &tmB, kb * KELEMS, t * BN, full(stage));
@@ -170,14 +170,14 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
             }
         }
     } else if (warp == CPRODUCER) {
-        if (lane == 0) {  // ------------------------------ class-value tile producer
+        if (elect_one()) {  // ------------------------------ class-value tile producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmV)) : "memory");
             const bool has_sb = p.sb != nullptr;
             uint32_t ph = 0, last = 0;
             bool any = false, ab = false;
             for (int64_t mt = blockIdx.x; mt < num_m_tiles && !ab; mt += gridDim.x)
                 for (int t = 0; t < p.nt; t++) {
-                    if (!mbar_wait(b2empty, ph ^ 1, abort_flag)) { ab = true; break; }
+                    if (!mbar_wait_fast(b2empty, ph ^ 1, abort_flag)) { ab = true; break; }
                     mbar_expect_tx(b2full, (uint32_t)(F16_B2_BYTES + (has_sb ? F16_SB_BYTES : 0)));
 #pragma unroll
                     for (int a = 0; a < 4; a++)   // 64 BF16 of K per atom
@@ -193,7 +193,7 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
             }
         }
     } else if (warp == ISSUER) {
-        if (lane == 0) {  // ------------------------------ MMA1 issuer (encode)
+        if (elect_one()) {  // ------------------------------ MMA1 issuer (encode)
             const uint32_t id1 = idesc_n<ENC>(BN);
             const uint64_t da0 = sdesc(su32(sA)), db0 = sdesc(su32(sB));
             const uint32_t full0 = full(0), empty0 = empty(0);   // stage s: + 8 * s
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
             while (!mbar_try(done_bar, 0) && gtimer() - t0 < 100000000ull) {}
         }
     } else if (warp == ISSUER2) {
-        if (lane == 0) {  // ------------------------------ MMA2 issuer (the tile's cosine partials)
+        if (elect_one()) {  // ------------------------------ MMA2 issuer (the tile's cosine partials)
             const uint32_t id2 = idesc_n<HDC_ENC_BF16>(F16_CP);
             uint32_t a2ph = 0, b2ph = 0;   // a2ph: the parity of both accumulators' a2full, flipped per pair
             int acc = 0;

@@ -178,7 +178,7 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == PRODUCER) {
-        if (lane == 0) {  // ------------------------------ A / B stage producer
+        if (elect_one()) {  // ------------------------------ A / B stage producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
             int stage = 0;
@@ -197,7 +197,7 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
                                                                  (uint32_t)(((it - 1) >> 1) & 1), abort_flag);
                             if (!okq) { ab = true; break; }
                         }
-                        if (!mbar_wait(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
+                        if (!mbar_wait_fast(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
                         mbar_expect_tx(full(stage), H_STAGE_BYTES);
                         const int ay = QIN ? (int)((blockIdx.x * 2 + (it & 1)) * BM) : (int)(mt * BM);
                         tma_load_2d(su32(sA + stage * HA_BYTES), &tmA, kb * KELEMS, ay, full(stage));
@@ -215,14 +215,14 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
             }
         }
     } else if (warp == CPRODUCER) {
-        if (lane == 0) {  // ------------------------------ class-sign producer
+        if (elect_one()) {  // ------------------------------ class-sign producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmS)) : "memory");
             uint32_t ph = 0, last = 0;
             bool any = false, ab = false;
             const uint32_t bytes = 2u * (uint32_t)p.Cp * 128u;
             for (int64_t mt = blockIdx.x; mt < num_m_tiles && !ab; mt += gridDim.x)
                 for (int t = 0; t < p.nt; t++) {
-                    if (!mbar_wait(b2empty, ph ^ 1, abort_flag)) { ab = true; break; }
+                    if (!mbar_wait_fast(b2empty, ph ^ 1, abort_flag)) { ab = true; break; }
                     mbar_expect_tx(b2full, bytes);
                     tma_load_2d(su32(sB2), &tmS, t * HBN, 0, b2full);
                     tma_load_2d(su32(sB2 + p.Cp * 128), &tmS, t * HBN + 128, 0, b2full);
@@ -236,7 +236,7 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
             }
         }
     } else if (warp == ISSUER) {
-        if (lane == 0) {  // ------------------------------ MMA1 issuer (encode)
+        if (elect_one()) {  // ------------------------------ MMA1 issuer (encode)
             const uint32_t id1 = idesc_n<ENC>(HBN);
             const uint64_t da0 = sdesc(su32(sA)), db0 = sdesc(su32(sB));
             const uint32_t full0 = full(0), empty0 = empty(0);   // stage s: + 8 * s
@@ -271,7 +271,7 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
             while (!mbar_try(done_bar, 0) && gtimer() - t0 < 100000000ull) {}
         }
     } else if (warp == ISSUER2) {
-        if (lane == 0) {  // ------------------------------ MMA2 issuer: D2 (+)= signs . class signs, K = 192
+        if (elect_one()) {  // ------------------------------ MMA2 issuer: D2 (+)= signs . class signs, K = 192
             const uint32_t id2 = idesc_n<HDC_ENC_FP8_E4M3>(p.Cp);
             uint32_t a2ph = 0, b2ph = 0, d2ph = 0;   // a2ph: both accumulators' parity, flipped per pair
             int acc = 0;

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     };
 
     if (warp == HP_ISSUER) {
-        if (lane == 0) {  // ------------------------------ MMA issuer
+        if (elect_one()) {  // ------------------------------ MMA issuer
             const uint32_t id = idesc_n<HDC_ENC_FP8_E4M3>(p.R);
             const uint64_t db0 = sdesc(su32(sB));
             int buf = 0, slot = 0, d2 = 0;
@@ -308,7 +308,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             while (!mbar_try(done_bar, 0) && gtimer() - t0 < 100000000ull) {}
         }
     } else if (warp == HP_QPROD || warp == HP_BPROD) {
-        if (lane == 0 && (PRE || warp == HP_QPROD)) {  // ---- TMA producers
+        if ((PRE || warp == HP_QPROD) && elect_one()) {  // ---- TMA producers
             const bool isq = warp == HP_QPROD;
             const int nslots = isq ? HP_QB : p.nbs;
             int slot = 0;

@@ -121,6 +121,19 @@ struct Params {
 // ------------------------------------------------------------ PTX wrappers
 __device__ __forceinline__ uint32_t su32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
+// One lane of a converged warp, chosen so that the compiler knows the code
+// below it has a single thread: the operands of the tcgen05 and TMA
+// instructions then live in uniform registers.  Under `if (lane == 0)` they
+// were moved there one by one before every instruction: a loop of MMAs issued
+// one per 117 cycles whatever its size, where N = 112 takes the tensor pipe 56
+// and N = 16 eight (measured: 56.2 and 9.3 cycles with this form).
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 __device__ __forceinline__ unsigned long long gtimer()
 {
     unsigned long long t;
@@ -460,7 +473,7 @@ __global__ void __launch_bounds__(num_threads(EWG, QIN), 1)
     const uint32_t tmem = *tmem_slot;
 
     if (warp == PRODUCER) {
-        if (lane == 0) {  // ---------------------------------- TMA producer
+        if (elect_one()) {  // ---------------------------------- TMA producer
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmA)) : "memory");
             asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmB)) : "memory");
             if (CLASSIFY) asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmC)) : "memory");
@@ -483,7 +496,7 @@ __global__ void __launch_bounds__(num_threads(EWG, QIN), 1)
                         if (!okq) { ab = true; break; }
                     }
                     if (CLASSIFY) {  // this dim tile's class words: C rows x 8 words (zeros past W)
-                        if (!mbar_wait(cempty(cb), cph ^ 1, abort_flag)) { ab = true; break; }
+                        if (!mbar_wait_fast(cempty(cb), cph ^ 1, abort_flag)) { ab = true; break; }
                         mbar_expect_tx(cfull(cb), (uint32_t)p.C * 32u);
                         tma_load_2d(su32(sCls + cb * CLS_BYTES), &tmC, nt * 8, 0, cfull(cb));
                         c_issued |= 1u << cb;
@@ -491,7 +504,7 @@ __global__ void __launch_bounds__(num_threads(EWG, QIN), 1)
                         if (++cb == CBUF) { cb = 0; cph ^= 1; }
                     }
                     for (int kb = 0; kb < p.num_kb; kb++) {
-                        if (!mbar_wait(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
+                        if (!mbar_wait_fast(empty(stage), phase ^ 1, abort_flag)) { ab = true; break; }
                         mbar_expect_tx(full(stage), STAGE_BYTES);
                         const int ay = QIN ? (int)((blockIdx.x * 2 + (it & 1)) * BM) : (int)(mt * BM);
                         tma_load_2d(su32(sA + stage * A_BYTES), &tmA, kb * KELEMS, ay, full(stage));
@@ -516,7 +529,7 @@ __global__ void __launch_bounds__(num_threads(EWG, QIN), 1)
             }
         }
     } else if (warp == ISSUER) {
-        if (lane == 0) {  // ---------------------------------- MMA issuer
+        if (elect_one()) {  // ---------------------------------- MMA issuer
             const uint32_t id = idesc<ENC>();
             const uint64_t da0 = sdesc(su32(sA)), db0 = sdesc(su32(sB));
             const uint32_t full0 = full(0), empty0 = empty(0);   // stage s: + 8 * s
