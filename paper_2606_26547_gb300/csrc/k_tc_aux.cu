@@ -140,11 +140,11 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
     p.S = pl.S;
     // shared memory: the query ring, the class atoms, barriers; at least 120 KB
     // so that no second CTA shares the SM and waits for its TMEM columns
-    const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::HP_TAIL, atom = (size_t)R * 128;
+    const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::hp_tail(pl.mt), atom = (size_t)R * 128;
     size_t nbs = (227 * 1024 - fixed) / atom;
     if (nbs > (size_t)tc::HP_NBS_MAX) nbs = tc::HP_NBS_MAX;
     p.nbs = (int)nbs;
-    size_t smem = fixed + (signs ? nbs * atom : 4 * atom + (size_t)((W + 3) & ~3) * 4);
+    size_t smem = fixed + (signs ? nbs * atom : tc::hp_nab(pl.mt, false) * atom + (size_t)((W + 3) & ~3) * 4);
     if (smem < 120 * 1024) smem = 120 * 1024;
     auto k = pl.mt == 2 ? (signs ? tc::tc_hamming_packed_kernel<2, true> : tc::tc_hamming_packed_kernel<2, false>)
                         : (signs ? tc::tc_hamming_packed_kernel<1, true> : tc::tc_hamming_packed_kernel<1, false>);

@@ -16,18 +16,20 @@
 //
 // One CTA per SM, persistent over units of MT x 128 query rows (MT = 2 up to
 // 128 class rows: the class bytes, R x D per unit, are the larger stream).
-// Roles (19 warps):
-//   warps 0-7   expand: a thread takes 256 dims (MT = 2: a row each) or 128
-//               dims (MT = 1: a row's half) of every 256-dim tile from the
-//               staged query words and writes them into its own TMEM lane
-//               (tcgen05.st), double buffered; operand A of the MMAs;
-//   warps 8-15  epilogue: D2 -> distances and arg-min, while the next unit's
-//               tiles accumulate into the other D2 (R <= 64);
-//   warp 16     TMA producer of the packed query words, 1,024 dims x MT x 128
+// Roles (27 warps):
+//   warps 0-15  expand: a thread takes its row's 128 dims of an atom (MT = 2:
+//               every second atom; MT = 1: every fourth) from the staged query words and writes them into its own
+//               TMEM lane (tcgen05.st): operand A of the MMAs, a ring of NAB
+//               atom buffers.  The bytes are formed before the wait for the
+//               buffer, so only the store and the MMAs are in its chain;
+//   warps 16-23 epilogue: D2 -> distances and arg-min, while the next unit's
+//               atoms accumulate into the other D2 (R <= 64); distances leave
+//               through shared memory as runs of a row;
+//   warp 24     TMA producer of the packed query words, 1,024 dims x MT x 128
 //               rows per copy (whole 128-byte lines), a ring of HP_QB chunks;
-//   warp 17     PRE: TMA producer of the class bytes (atoms of R rows x 128
+//   warp 25     PRE: TMA producer of the class bytes (atoms of R rows x 128
 //               dims) into a ring of p.nbs slots;
-//   warp 18     MMA issuer.
+//   warp 26     MMA issuer.
 // PRE: the class rows come already expanded (Cp rows of ldcs bytes, from
 // launch_class_bytes into the caller's workspace).  Without it the expanding
 // warps also expand the class words of every tile into two shared-memory
@@ -39,7 +41,7 @@
 // finished by the ranks in turn.
 //
 // TMEM (512 columns): D2 in columns 0..255 (MT x RS columns a buffer, RS = R
-// rounded up to 32), the two query buffers of MT x 64 columns from 256.
+// rounded up to 32), the NAB query buffers of MT x 32 columns from 256.
 // Every wait is bounded as in the encoder.
 //
 // What bounds it, and the form before: see launch_hamming_packed.
@@ -49,10 +51,10 @@
 namespace hdc {
 namespace tc {
 
-constexpr int HP_EXP = 256;                    // expanding threads (warps 0-7)
-constexpr int HP_EPI0 = HP_EXP / 32;           // first of the eight epilogue warps
-constexpr int HP_QPROD = 16, HP_BPROD = 17, HP_ISSUER = 18;
-constexpr int HP_THREADS = 19 * 32;
+constexpr int HP_EXPW = 16;                    // expanding warps (0-15)
+constexpr int HP_EPI0 = HP_EXPW;               // first of the eight epilogue warps
+constexpr int HP_QPROD = HP_EXPW + 8, HP_BPROD = HP_EXPW + 9, HP_ISSUER = HP_EXPW + 10;
+constexpr int HP_THREADS = (HP_EXPW + 11) * 32;
 constexpr int HP_CMAX = 256;
 constexpr int HP_MAX_W = 4096;                 // words of a packed row (D <= 131072)
 constexpr int HP_QB = 3;                       // query chunks in the ring
@@ -60,9 +62,13 @@ constexpr int HP_CHUNK = 4;                    // 256-dim tiles per query chunk 
 constexpr int HP_NBS_MAX = 16;                 // most class-atom slots
 constexpr int HP_SMAX = 8;                     // most CTAs a unit's dims are split over
 constexpr uint32_t HP_ACOL = 256;              // first TMEM column of the query buffers
-// qfull[QB], qempty[QB], bfull[NBS], bempty[NBS], afull[2], aempty[2], d2full[2], d2empty[2], done
-constexpr int HP_NUM_BARS = 2 * HP_QB + 2 * HP_NBS_MAX + 9;
-constexpr int HP_TAIL = HP_NUM_BARS * 8 + 16 + 2 * HP_CMAX * 4;   // barriers, TMEM slot, abort flag, group counts
+constexpr int HP_NAB_MAX = 8;                  // query-atom buffers: 4, or 8 with MT = 1 and PRE
+__host__ __device__ constexpr int hp_nab(int mt, bool pre) { return mt == 1 && pre ? 8 : 4; }
+// qfull[QB], qempty[QB], bfull[NBS], bempty[NBS], afull[NAB], aempty[NAB], d2full[2], d2empty[2], done
+constexpr int HP_NUM_BARS = 2 * HP_QB + 2 * HP_NBS_MAX + 2 * HP_NAB_MAX + 5;
+constexpr int HP_OUT = 32 * 33 * 4;            // an epilogue warp's 32 x 32 distances, padded rows
+// epilogue staging, barriers, TMEM slot, abort flag
+__host__ __device__ constexpr int hp_tail(int mt) { return 4 * mt * HP_OUT + HP_NUM_BARS * 8 + 16; }
 
 __host__ __device__ constexpr int hp_q_bytes(int mt) { return HP_QB * mt * 128 * 128; }
 
@@ -112,31 +118,21 @@ __device__ __forceinline__ void hp_tmem_st32(uint32_t taddr, const uint32_t (&r)
         : "memory");
 }
 
-// 128 dims (four words) of a row into 32 TMEM columns of its lane.
-__device__ __forceinline__ void hp_expand_tmem(uint32_t taddr, const uint4 w)
-{
-    const uint32_t ws[4] = {w.x, w.y, w.z, w.w};
-    uint32_t b[32];
-#pragma unroll
-    for (int i = 0; i < 4; i++)
-#pragma unroll
-        for (int j = 0; j < 8; j++) b[8 * i + j] = hp_signs(ws[i], j);
-    hp_tmem_st32(taddr, b);
-}
-
-// 128 dims (four words) of class row r into its 128-byte row of a K atom
-// (128-byte swizzle), zero outside the mask words.
-__device__ __forceinline__ void hp_expand_row(uint8_t *atom, int r, const uint4 w, const uint4 m)
+// NW words of class row r into its 128-byte row of a K atom (128-byte
+// swizzle), from 16-byte piece `p0` on; zero outside the mask words.  A class
+// row past C has zero words: its products are never read.
+template <int NW>
+__device__ __forceinline__ void hp_expand_row(uint8_t *atom, int r, int p0, const uint4 w, const uint4 m)
 {
     uint8_t *row = atom + r * 128;
     const uint32_t ws[4] = {w.x, w.y, w.z, w.w}, ms[4] = {m.x, m.y, m.z, m.w};
 #pragma unroll
-    for (int i = 0; i < 4; i++) {
+    for (int i = 0; i < NW; i++) {
         uint32_t b[8];
 #pragma unroll
         for (int j = 0; j < 8; j++) b[j] = hp_signs(ws[i], j) & hp_mask(ms[i], j);
-        *reinterpret_cast<uint4 *>(row + (((2 * i) ^ (r & 7)) * 16)) = make_uint4(b[0], b[1], b[2], b[3]);
-        *reinterpret_cast<uint4 *>(row + (((2 * i + 1) ^ (r & 7)) * 16)) = make_uint4(b[4], b[5], b[6], b[7]);
+        *reinterpret_cast<uint4 *>(row + (((p0 + 2 * i) ^ (r & 7)) * 16)) = make_uint4(b[0], b[1], b[2], b[3]);
+        *reinterpret_cast<uint4 *>(row + (((p0 + 2 * i + 1) ^ (r & 7)) * 16)) = make_uint4(b[4], b[5], b[6], b[7]);
     }
 }
 
@@ -165,10 +161,12 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     constexpr int UROWS = MT * BM;                               // query rows of a unit
     constexpr int QCH = UROWS * 128;                             // bytes of a query chunk
     uint8_t *sQ = smem;
-    uint8_t *sB = smem + hp_q_bytes(MT);                         // PRE: nbs atoms; else two tiles of two atoms
+    constexpr int NAB = hp_nab(MT, PRE);
+    uint8_t *sB = smem + hp_q_bytes(MT);                         // class atoms: nbs, or one per query buffer
     const int atom_bytes = p.R * 128;
-    uint32_t *smask = reinterpret_cast<uint32_t *>(sB + (size_t)(PRE ? p.nbs : 4) * atom_bytes);   // W words (not PRE)
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smask + (PRE ? 0 : ((p.W + 3) & ~3)));
+    int32_t *s_out = reinterpret_cast<int32_t *>(sB + (size_t)(PRE ? p.nbs : NAB) * atom_bytes);   // 4 * MT x HP_OUT
+    uint64_t *bars = reinterpret_cast<uint64_t *>(s_out + 4 * MT * (HP_OUT / 4));
+    uint32_t *smask = reinterpret_cast<uint32_t *>(bars + HP_NUM_BARS + 1);   // W words (not PRE)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(bars + HP_NUM_BARS);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(tmem_slot + 1);
     auto qfull = [&](int b) { return su32(bars + b); };
@@ -177,10 +175,10 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     auto bempty = [&](int b) { return su32(bars + 2 * HP_QB + HP_NBS_MAX + b); };
     constexpr int X = 2 * HP_QB + 2 * HP_NBS_MAX;
     auto afull = [&](int b) { return su32(bars + X + b); };
-    auto aempty = [&](int b) { return su32(bars + X + 2 + b); };
-    auto d2full = [&](int b) { return su32(bars + X + 4 + b); };
-    auto d2empty = [&](int b) { return su32(bars + X + 6 + b); };
-    const uint32_t done_bar = su32(bars + X + 8);
+    auto aempty = [&](int b) { return su32(bars + X + HP_NAB_MAX + b); };
+    auto d2full = [&](int b) { return su32(bars + X + 2 * HP_NAB_MAX + b); };
+    auto d2empty = [&](int b) { return su32(bars + X + 2 * HP_NAB_MAX + 2 + b); };
+    const uint32_t done_bar = su32(bars + X + 2 * HP_NAB_MAX + 4);
 
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int RS = (p.R + 31) & ~31;                 // D2 columns of one 128-row tile
@@ -191,20 +189,22 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     const int64_t u0 = blockIdx.x / S, ustep = gridDim.x / S;
     const int chunks = (p.nt + HP_CHUNK - 1) / HP_CHUNK;
     const int ch0 = chunks * rank / S, ch1 = chunks * (rank + 1) / S;   // this rank's query chunks
-    auto chunk_tiles = [&](int ch) { return min(HP_CHUNK, p.nt - ch * HP_CHUNK); };
+    auto chunk_atoms = [&](int ch) { return 2 * min(HP_CHUNK, p.nt - ch * HP_CHUNK); };
 
     if (tid == 0) {
         for (int b = 0; b < HP_QB; b++) {
             mbar_init(qfull(b), 1);
-            mbar_init(qempty(b), HP_EXP / 32);
+            mbar_init(qempty(b), HP_EXPW);
         }
         for (int b = 0; b < HP_NBS_MAX; b++) {
             mbar_init(bfull(b), 1);
             mbar_init(bempty(b), 1);
         }
-        for (int b = 0; b < 2; b++) {
-            mbar_init(afull(b), HP_EXP / 32);
+        for (int b = 0; b < NAB; b++) {
+            mbar_init(afull(b), 4 * MT);
             mbar_init(aempty(b), 1);
+        }
+        for (int b = 0; b < 2; b++) {
             mbar_init(d2full(b), 1);
             mbar_init(d2empty(b), 4 * MT);
         }
@@ -225,46 +225,55 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     tc_fence_after();
     const uint32_t tmem = *tmem_slot;
 
-    // Distances and arg-min of one row from its R dot products, read 32
-    // columns at a time by `cols(j, v)`.
-    auto finish = [&](int64_t row, auto cols) {
-        const bool valid = row < p.N;
+    // Distances and arg-min of the 32 rows from `row0` on (this lane's is
+    // row0 + lane) from their R dot products, read 32 columns at a time by
+    // cols(j, v); `out`: the warp's staging for the distances.
+    auto finish = [&](int64_t row0, int32_t *out, auto cols) {
         int best = 0;
         float bd = -3.0e38f;   // largest dot = smallest distance; ascending c: lowest class on ties
-        const bool vec = p.dists && p.C % 4 == 0 && (reinterpret_cast<uintptr_t>(p.dists) & 15) == 0;
+        const bool vec = p.C % 4 == 0 && (reinterpret_cast<uintptr_t>(p.dists) & 15) == 0;
+        const int nrow = (int)min((int64_t)32, p.N - row0);   // rows of this warp below N (may be <= 0)
         for (int j = 0; j * 32 < p.R; j++) {
             uint32_t v[32];
             cols(j, v);
+            const int nc = min(32, p.C - j * 32);
 #pragma unroll
             for (int i = 0; i < 32; i++) {
                 const float d = __uint_as_float(v[i]);
-                if (j * 32 + i < p.C && d > bd) { bd = d; best = j * 32 + i; }
+                if (i < nc && d > bd) { bd = d; best = j * 32 + i; }
             }
-            if (p.dists && valid) {
-                int32_t *o = p.dists + row * p.C + j * 32;
+            if (p.dists) {
 #pragma unroll
                 for (int i = 0; i < 32; i++) v[i] = (uint32_t)((p.kept - (int)__uint_as_float(v[i])) / 2);
-                if (vec) {
+                if (vec) {   // 16 bytes a store: 10^5 x 256 classes 23 us of distances (41 us staged)
+                    int32_t *o = p.dists + (row0 + lane) * p.C + j * 32;
 #pragma unroll
                     for (int i = 0; i < 32; i += 4)
-                        if (j * 32 + i < p.C)
+                        if (i < nc && lane < nrow)
                             *reinterpret_cast<uint4 *>(o + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                } else {
+                } else {     // 10^6 x 33 classes: 44 us (125 us of single words)
+                    __syncwarp();
 #pragma unroll
                     for (int i = 0; i < 32; i++)
-                        if (j * 32 + i < p.C) o[i] = (int32_t)v[i];
+                        if (i < nc) out[lane * 33 + i] = (int32_t)v[i];
+                    __syncwarp();
+                    int32_t *o = p.dists + row0 * p.C + j * 32 + lane;
+                    if (lane < nc)
+#pragma unroll 8
+                        for (int r = 0; r < 32; r++)
+                            if (r < nrow) o[(int64_t)r * p.C] = out[r * 33 + lane];
                 }
             }
         }
-        if (valid) p.labels[row] = best;
+        if (lane < nrow) p.labels[row0 + lane] = best;
     };
 
     if (warp == HP_ISSUER) {
         if (elect_one()) {  // ------------------------------ MMA issuer
             const uint32_t id = idesc_n<HDC_ENC_FP8_E4M3>(p.R);
             const uint64_t db0 = sdesc(su32(sB));
-            int buf = 0, slot = 0, d2 = 0;
-            uint32_t aph = 0, bph = 0, d2ph[2] = {0, 0};
+            int slot = 0, d2 = 0;
+            uint32_t g = 0, bph = 0, d2ph[2] = {0, 0};   // g: atoms so far
             bool ab = false;
             for (int64_t u = u0; u < units && !ab; u += ustep) {
                 if (!mbar_wait_fast(d2empty(d2), d2ph[d2] ^ 1, abort_flag)) { ab = true; break; }
@@ -272,31 +281,26 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                 const uint32_t dcol = tmem + (uint32_t)(d2 * MT * RS);
                 uint32_t accum = 0;
                 for (int ch = ch0; ch < ch1 && !ab; ch++) {
-                    const int ntl = chunk_tiles(ch);
-                    for (int t = 0; t < ntl; t++) {
-                        if (!mbar_wait_fast(afull(buf), aph, abort_flag)) { ab = true; break; }
-                        const uint32_t acol = tmem + HP_ACOL + (uint32_t)(buf * MT * 64);
+                    const int na = chunk_atoms(ch);
+                    for (int a = 0; a < na; a++, g++) {   // an atom: four 32-byte K steps of every query tile
+                        const int buf = g % NAB;
+                        if (!mbar_wait_fast(afull(buf), (g / NAB) & 1, abort_flag)) { ab = true; break; }
+                        if (PRE && !mbar_wait_fast(bfull(slot), bph, abort_flag)) { ab = true; break; }
+                        tc_fence_after();
+                        const uint32_t acol = tmem + HP_ACOL + (uint32_t)(buf * MT * 32);
+                        const uint64_t db = db0 + (uint64_t)(PRE ? slot : buf) * (uint64_t)(atom_bytes >> 4);
 #pragma unroll
-                        for (int a = 0; a < 2; a++) {   // two atoms of four 32-byte K steps
-                            if (PRE && !mbar_wait_fast(bfull(slot), bph, abort_flag)) { ab = true; break; }
-                            tc_fence_after();
-                            const int at = PRE ? slot : buf * 2 + a;
-                            const uint64_t db = db0 + (uint64_t)at * (uint64_t)(atom_bytes >> 4);
+                        for (int m = 0; m < MT; m++)
 #pragma unroll
-                            for (int m = 0; m < MT; m++)
-#pragma unroll
-                                for (int k = 0; k < 4; k++)
-                                    h_mma_ts_fp8(dcol + (uint32_t)(m * RS), acol + (uint32_t)(m * 64 + a * 32 + 8 * k),
-                                                 db + 2 * k, id, accum | (uint32_t)k);
-                            accum = 1;
-                            if (PRE) {
-                                mma_commit(bempty(slot));
-                                if (++slot == p.nbs) { slot = 0; bph ^= 1; }
-                            }
-                        }
-                        if (ab) break;
+                            for (int k = 0; k < 4; k++)
+                                h_mma_ts_fp8(dcol + (uint32_t)(m * RS), acol + (uint32_t)(m * 32 + 8 * k), db + 2 * k, id,
+                                             accum | (uint32_t)k);
+                        accum = 1;
                         mma_commit(aempty(buf));
-                        if (++buf == 2) { buf = 0; aph ^= 1; }
+                        if (PRE) {
+                            mma_commit(bempty(slot));
+                            if (++slot == p.nbs) { slot = 0; bph ^= 1; }
+                        }
                     }
                 }
                 if (ab) break;
@@ -316,7 +320,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             bool ab = false;
             for (int64_t u = u0; u < units && !ab; u += ustep)
                 for (int ch = ch0; ch < ch1 && !ab; ch++) {
-                    const int n = isq ? 1 : 2 * chunk_tiles(ch);   // a query chunk, or the atoms of its tiles
+                    const int n = isq ? 1 : chunk_atoms(ch);   // a query chunk, or its class atoms
                     for (int a = 0; a < n; a++) {
                         const uint32_t fb = isq ? qfull(slot) : bfull(slot);
                         if (!mbar_wait_fast(isq ? qempty(slot) : bempty(slot), ph ^ 1, abort_flag)) { ab = true; break; }
@@ -343,75 +347,91 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                     }
         }
     } else if (warp < HP_EPI0) {  // ---------------------- expanding warps
-        const int urow = MT == 2 ? tid : (tid & (BM - 1));      // row of the unit
-        const int half = MT == 2 ? 0 : tid >> 7;                // MT = 1: this thread's 128 dims of a tile
-        const uint32_t tlane = (uint32_t)((warp & 3) * 32) << 16;
-        const uint32_t tcol = tmem + tlane + HP_ACOL + (uint32_t)(MT == 2 ? (warp >> 2) * 64 : half * 32);
-        int buf = 0, qs = 0;
-        uint32_t aph = 0, qph = 0;
+        const int urow = tid % UROWS;                           // row of the unit
+        // every AS-th atom of the CTA, from number `grp` on: AS <= NAB, so a
+        // buffer's phase is never two generations behind the one awaited
+        constexpr int AS = HP_EXPW / (4 * MT);
+        static_assert(AS <= NAB, "an expanding warp's next atom is at most one round of the buffers away");
+        const uint32_t grp = (uint32_t)(warp / (4 * MT));
+        const uint32_t tcol = tmem + ((uint32_t)((warp & 3) * 32) << 16) + HP_ACOL + (uint32_t)(urow / BM * 32);
+        int qs = 0;
+        uint32_t qph = 0, gch = 0;   // gch: the chunk's first atom, numbered in the CTA
         bool ab = false;
-        // class words (not PRE): items i = tid and tid + 256, class i % R, half i / R of the tile
-        auto class_words = [&](int i, int t) {
-            const int c = i % p.R, wc = t * 8 + (i / p.R) * 4;
-            return (i < 2 * p.R && c < p.C && wc < p.W)
-                       ? __ldg(reinterpret_cast<const uint4 *>(p.cls + (int64_t)c * p.W + wc))
-                       : make_uint4(0, 0, 0, 0);
+        // class words (not PRE) of this thread in atom t: row c0, its words
+        // [2 * part, 2 * part + 2) with MT = 2 (2 R items), rows c0 and
+        // c0 + 128 whole with MT = 1
+        const int c0 = MT == 2 ? urow % p.R : urow, part = MT == 2 ? urow / p.R : 0;
+        auto class_words = [&](int c, int t) {
+            const bool ok = part < 2 && c < p.C && t * 4 < p.W;
+            const uint32_t *w = p.cls + (int64_t)(ok ? c : 0) * p.W + (ok ? t * 4 : 0);
+            if (!ok) return make_uint4(0, 0, 0, 0);
+            if (MT == 1) return __ldg(reinterpret_cast<const uint4 *>(w));
+            const uint2 h = __ldg(reinterpret_cast<const uint2 *>(w + part * 2));
+            return make_uint4(h.x, h.y, 0, 0);
         };
+        const int tu0 = ch0 * 2 * HP_CHUNK, tun = min(ch1 * 2 * HP_CHUNK, 2 * p.nt) - tu0;   // a unit's atoms
+        uint4 cn0, cn1;   // class words of this warp's next atom
+        if (!PRE) {
+            cn0 = class_words(c0, tu0 + (int)grp % tun);
+            if (MT == 1) cn1 = class_words(c0 + 128, tu0 + (int)grp % tun);
+        }
         for (int64_t u = u0; u < units && !ab; u += ustep) {
-            uint4 cn0, cn1;
-            if (!PRE) {
-                cn0 = class_words(tid, ch0 * HP_CHUNK);
-                cn1 = class_words(tid + HP_EXP, ch0 * HP_CHUNK);
-            }
             for (int ch = ch0; ch < ch1 && !ab; ch++) {
                 const bool okq = mbar_wait(qfull(qs), qph, abort_flag);
                 if (!__all_sync(0xffffffffu, okq)) { ab = true; break; }
                 const uint8_t *qrow = sQ + qs * QCH + urow * 128;
-                const int ntl = chunk_tiles(ch);
-                for (int tl = 0; tl < ntl; tl++) {
-                    const int t = ch * HP_CHUNK + tl;
-                    const uint4 w0 = *reinterpret_cast<const uint4 *>(qrow + (((tl * 2 + half) ^ (urow & 7)) << 4));
-                    uint4 w1;
-                    if (MT == 2) w1 = *reinterpret_cast<const uint4 *>(qrow + (((tl * 2 + 1) ^ (urow & 7)) << 4));
-                    if (tl == ntl - 1) {   // the chunk's words are in registers: its slot may be refilled
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(qempty(qs));
-                    }
+                const int na = chunk_atoms(ch);
+                const int a0 = (int)((grp - gch) % (uint32_t)AS);
+                if (a0 >= na && lane == 0) mbar_arrive(qempty(qs));
+                for (int a = a0; a < na; a += AS) {
+                    const int t = ch * 2 * HP_CHUNK + a;
+                    const uint32_t g = gch + (uint32_t)a;
+                    const uint4 qw = *reinterpret_cast<const uint4 *>(qrow + ((a ^ (urow & 7)) << 4));
+                    const uint32_t ws[4] = {qw.x, qw.y, qw.z, qw.w};
+                    uint32_t b[32];
+#pragma unroll
+                    for (int i = 0; i < 4; i++)
+#pragma unroll
+                        for (int j = 0; j < 8; j++) b[8 * i + j] = hp_signs(ws[i], j);
                     const uint4 cw0 = cn0, cw1 = cn1;
-                    if (!PRE && t + 1 < ch1 * HP_CHUNK && t + 1 < p.nt) {
-                        cn0 = class_words(tid, t + 1);
-                        cn1 = class_words(tid + HP_EXP, t + 1);
+                    if (!PRE) {   // AS atoms on, in this unit or a following one
+                        const int tn = tu0 + (t - tu0 + AS) % tun;
+                        cn0 = class_words(c0, tn);
+                        if (MT == 1) cn1 = class_words(c0 + 128, tn);
                     }
-                    const bool oke = mbar_wait(aempty(buf), aph ^ 1, abort_flag);   // the MMAs of this buffer's last use
+                    const int buf = g % NAB;
+                    const bool oke = mbar_wait_fast(aempty(buf), ((g / NAB) & 1) ^ 1, abort_flag);   // its last MMAs
                     if (!__all_sync(0xffffffffu, oke)) { ab = true; break; }
                     tc_fence_after();
-                    const uint32_t ta = tcol + (uint32_t)(buf * MT * 64);
-                    hp_expand_tmem(ta, w0);
-                    if (MT == 2) hp_expand_tmem(ta + 32, w1);
+                    __syncwarp();   // converged for the warp-wide store
+                    hp_tmem_st32(tcol + (uint32_t)(buf * MT * 32), b);
                     if (!PRE) {
-#pragma unroll
-                        for (int ii = 0; ii < 2; ii++) {
-                            const int i = tid + ii * HP_EXP;
-                            if (i < 2 * p.R) {
-                                const int c = i % p.R, h = i / p.R, wc = t * 8 + h * 4;
-                                const uint4 mc = (c < p.C && wc < p.W) ? *reinterpret_cast<const uint4 *>(smask + wc)
-                                                                       : make_uint4(0, 0, 0, 0);
-                                hp_expand_row(sB + (buf * 2 + h) * atom_bytes, c, ii ? cw1 : cw0, mc);
-                            }
+                        const uint4 m = t * 4 < p.W ? *reinterpret_cast<const uint4 *>(smask + t * 4) : make_uint4(0, 0, 0, 0);
+                        uint8_t *at = sB + buf * atom_bytes;
+                        if (MT == 2) {
+                            if (part < 2) hp_expand_row<2>(at, c0, part * 4, cw0, part ? make_uint4(m.z, m.w, 0, 0) : m);
+                        } else {
+                            if (c0 < p.R) hp_expand_row<4>(at, c0, 0, cw0, m);
+                            if (c0 + 128 < p.R) hp_expand_row<4>(at, c0 + 128, 0, cw1, m);
                         }
                         fence_async_smem();
-                        __syncwarp();
                     }
                     h_tmem_st_wait();   // the query columns landed before the MMAs read them
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(afull(buf));
-                    if (++buf == 2) { buf = 0; aph ^= 1; }
+                    // the chunk's slot is given back only here, past the store
+                    // that consumed its last words: ahead of the wait for the
+                    // buffer the loads could still be outstanding
+                    if (lane == 0) {
+                        mbar_arrive(afull(buf));
+                        if (a + AS >= na) mbar_arrive(qempty(qs));
+                    }
                 }
+                gch += (uint32_t)na;
                 if (++qs == HP_QB) { qs = 0; qph ^= 1; }
             }
         }
-    } else if (warp - HP_EPI0 < 4 * MT) {  // -------------- epilogue warps 8 .. 7 + 4 * MT
+    } else if (warp - HP_EPI0 < 4 * MT) {  // -------------- epilogue warps 16 .. 15 + 4 * MT
         const int e = warp - HP_EPI0;
         const uint32_t tlane = (uint32_t)((warp & 3) * 32) << 16;
         int d2 = 0;
@@ -422,7 +442,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             tc_fence_after();
             const uint32_t dcol = tmem + tlane + (uint32_t)((d2 * MT + (e >> 2)) * RS);
             if (S == 1) {
-                finish(u * UROWS + e * 32 + lane, [&](int j, uint32_t(&v)[32]) { tmem_ld32(dcol + (uint32_t)(j * 32), v); });
+                finish(u * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) { tmem_ld32(dcol + (uint32_t)(j * 32), v); });
             } else {   // this rank's partial sums, [column][row of the unit], over the rings (all consumed)
                 float *dump = reinterpret_cast<float *>(smem) + e * 32 + lane;
                 for (int j = 0; j * 32 < p.R; j++) {
@@ -446,7 +466,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         const int e = warp - HP_EPI0;
         if (e >= 0 && e < 4 * MT && e % S == rank && u0 < units) {
             const uint32_t base = su32(smem) + (uint32_t)(e * 32 + lane) * 4u;
-            finish(u0 * UROWS + e * 32 + lane, [&](int j, uint32_t(&v)[32]) {
+            finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) {
 #pragma unroll
                 for (int i = 0; i < 32; i++) {
                     float s = 0.f;

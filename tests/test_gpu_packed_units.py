@@ -48,3 +48,24 @@ def test_hamming_units(hdc, N, D, C, perf):
         assert np.array_equal(labels.cpu().numpy()[rows], orc.argmin(od))
         # every row: its label is the lowest class of its smallest distance
         assert torch.equal(labels.long(), dd.argmin(1))
+
+
+def unpack_pm1(words, D):
+    bits = (words[:, :, None] >> torch.arange(32, device=words.device, dtype=torch.int32)) & 1
+    return 1.0 - 2.0 * bits.reshape(words.shape[0], -1)[:, :D].float()
+
+
+@pytest.mark.parametrize("N,D,C", [(30000, 4096, 256), (80000, 8192, 100), (80000, 4096, 97), (80000, 4096, 40)])
+def test_hamming_units_every_row(hdc, N, D, C):
+    """Several units a CTA while the distances are written: every distance of
+    every row equals the +-1 product (sums of at most D ones: exact in FP32)."""
+    g = torch.Generator(device="cuda").manual_seed(C)
+    W = hdc.words(D)
+    q, c = (torch.randint(-2 ** 31, 2 ** 31 - 1, (n, W), generator=g, device="cuda", dtype=torch.int64).to(torch.int32)
+            for n in (N, C))
+    k = unpack_pm1(c, D)
+    ref = torch.cat([(D - unpack_pm1(q[r:r + 10000], D) @ k.t()) / 2 for r in range(0, N, 10000)]).to(torch.int32)
+    for use_ws in (True, False, True, False):
+        labels, dd = hdc.hamming_argmin(q, c, D, dists=True, use_ws=use_ws)
+        assert torch.equal(dd, ref)
+        assert torch.equal(labels.long(), ref.argmin(1))
