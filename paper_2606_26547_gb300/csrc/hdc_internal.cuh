@@ -202,6 +202,28 @@ int hamming_packed_ldcs(int W);
 cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *cls, int C, int W, int64_t D,
                                   int64_t s0, int64_t e0, int64_t stride, int32_t *labels, int32_t *dists,
                                   cudaStream_t st, uint8_t *signs = nullptr);
+// Cosine arg-max of packed rows against b-bit class values on the tensor
+// cores: vals holds C * P rows of hamming_packed_ldcs(W) bytes, the P base-16
+// digits of a class side by side, in the packed kernel's dim order (C * P <=
+// 256, P 1 or 2); score = dot / cnorm in FP64 (0 for a zero norm).
+cudaError_t launch_packed_cosine(const uint32_t *Q, int64_t N, int W, const uint8_t *vals, int C, int P,
+                                 const double *cnorm, int32_t *labels, double *scores, cudaStream_t st);
+// Configurations of the sweep in one pass over the packed rows H: digits[i]
+// base-16 digits a class value (0: class signs, Hamming), output entry out[i],
+// their class rows one after the other in vals (at most 256 rows in all);
+// sumsq[out * C + c] the sum of the squared class values.
+struct PackedSweep {
+    const uint32_t *H;
+    const int32_t *y;
+    int64_t N;
+    int W, C, ncfg;
+    uint8_t digits[HDC_SWEEP_MAX_STRIDES * HDC_SWEEP_MAX_BITS], out[HDC_SWEEP_MAX_STRIDES * HDC_SWEEP_MAX_BITS];
+    const uint8_t *vals;
+    const long long *sumsq;
+    int32_t *correct, *labels;
+};
+cudaError_t launch_packed_sweep(const PackedSweep &a, cudaStream_t st);
+
 // One block waiting, bounded by limit_ns, on a barrier nothing arrives on
 // (the expiry is reported through tc_read_status).
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st);

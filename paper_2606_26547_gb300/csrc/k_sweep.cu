@@ -17,6 +17,7 @@
 #include <math.h>
 
 #include "hdc_internal.cuh"
+#include "quant_math.cuh"
 
 namespace hdc {
 namespace {
@@ -265,6 +266,113 @@ __global__ void sweep_eval_kernel(const uint32_t *__restrict__ H, const int32_t 
     }
 }
 
+// ---- tensor-core route ------------------------------------------------------
+// Class values of every configuration as rows of E4M3 base-16 digits, zero
+// outside the entry's dims, in the packed kernel's dim order (word w's byte
+// 4j + k is dim 32w + j + 8k): row[i] + c * digits + q for configuration i,
+// class c, digit q.  The query rows are then expanded once for all of them.
+struct SweepRows {
+    int n;                  // configurations
+    int jb[MAXB * MAXS], entry[MAXB * MAXS], digits[MAXB * MAXS], row[MAXB * MAXS];
+};
+
+__device__ __forceinline__ uint32_t entry_mask(const SweepConf &cf, int i, int w);
+
+// A block takes one class and 1,024 dims (a thread four dims of one word),
+// after scanning all of the class's accumulators for its largest magnitude;
+// the squares of the kept values are added into sumsq (zeroed by the caller).
+// One block a class for everything took most of the time of a short sweep.
+constexpr int SPD = 1024;
+__global__ void __launch_bounds__(256) sweep_digits_kernel(const int32_t *__restrict__ acc, int D, int C, int ld,
+                                                           const __grid_constant__ SweepConf cf,
+                                                           const __grid_constant__ SweepRows rw,
+                                                           uint8_t *__restrict__ vals, long long *__restrict__ sumsq)
+{
+    __shared__ unsigned s_max;
+    __shared__ unsigned long long s_sq[MAXB * MAXS];
+    const int c = blockIdx.x, tid = threadIdx.x;
+    const int32_t *a = acc + (int64_t)c * D;
+    if (tid == 0) s_max = 0;
+    if (tid < MAXB * MAXS) s_sq[tid] = 0;
+    __syncthreads();
+    unsigned m = 0;   // |acc| < 2^31; -2^31 itself has magnitude 2^31 in 32 bits unsigned
+#pragma unroll 8
+    for (int d = tid; d < D; d += 256) {
+        const int v = __ldg(a + d);
+        m = max(m, v < 0 ? 0u - (unsigned)v : (unsigned)v);
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((tid & 31) == 0) atomicMax(&s_max, m);
+    __syncthreads();
+    const long long M = s_max;
+    const int w = blockIdx.y * (SPD / 32) + (tid >> 3), j = tid & 7;   // dims 32w + j + 8k, k = 0..3
+    long long x[4];
+#pragma unroll
+    for (int k = 0; k < 4; k++) {
+        const int d = w * 32 + j + 8 * k;
+        x[k] = d < D ? (long long)__ldg(a + d) : 0;
+    }
+    for (int jb = 0; jb < cf.nb; jb++) {
+        long long v[4];
+#pragma unroll
+        for (int k = 0; k < 4; k++) v[k] = w * 32 + j + 8 * k < D ? class_value(x[k], cf.bits[jb], M) : 0;
+        for (int f = 0; f < rw.n; f++) {
+            if (rw.jb[f] != jb) continue;
+            const uint32_t em = entry_mask(cf, rw.entry[f], w) >> j;
+            long long r[4], sq = 0;
+#pragma unroll
+            for (int k = 0; k < 4; k++) {
+                r[k] = (em >> (8 * k)) & 1u ? v[k] : 0;
+                sq += r[k] * r[k];
+            }
+            if (w * 32 < ld) {
+                uint32_t *o = reinterpret_cast<uint32_t *>(vals + (int64_t)(rw.row[f] + c * rw.digits[f]) * ld + w * 32) + j;
+                for (int q = 0; q < rw.digits[f]; q++) {
+                    float g[4];
+#pragma unroll
+                    for (int k = 0; k < 4; k++) {   // signed digits -8..7, the last one takes what is left
+                        const int dg = q == rw.digits[f] - 1 ? (int)r[k] : (int)((r[k] + 8) & 15) - 8;
+                        r[k] = (r[k] - dg) >> 4;
+                        g[k] = (float)dg;
+                    }
+                    o[(int64_t)q * (ld / 4)] = to_e4m3x4(g[0], g[1], g[2], g[3]);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+            if ((tid & 31) == 0 && sq) atomicAdd(&s_sq[f], (unsigned long long)sq);
+        }
+    }
+    __syncthreads();
+    if (tid < rw.n && s_sq[tid])
+        atomicAdd((unsigned long long *)sumsq + (int64_t)(rw.jb[tid] * cf.ns + rw.entry[tid]) * C + c, s_sq[tid]);
+}
+
+// Rows of the configurations, and whether the tensor-core route takes them:
+// every configuration's class rows fit one pass (256 rows), rows of at most
+// 4,096 words.
+bool sweep_rows(const SweepConf &cf, int C, int W, SweepRows *rw, int *total)
+{
+    rw->n = 0;
+    int64_t row = 0;
+    bool ok = W <= 4096;
+    for (int j = 0; j < cf.nb; j++) {
+        const int dg = cf.bits[j] == 0 ? 8 : cf.bits[j] == 8 ? 2 : 1;
+        if ((int64_t)C * dg > 256) ok = false;
+        for (int i = 0; i < cf.ns; i++) {
+            rw->jb[rw->n] = j;
+            rw->entry[rw->n] = i;
+            rw->digits[rw->n] = dg;
+            rw->row[rw->n] = (int)row;
+            rw->n++;
+            row += (int64_t)C * dg;
+            if (row > 1 << 20) ok = false;
+        }
+    }
+    *total = (int)row;
+    return ok;
+}
+
 bool is_pow2_le32(int s) { return s >= 1 && s <= 32 && (s & (s - 1)) == 0; }
 
 bool make_conf(const hdc_sweep_spec *sp, int64_t D, SweepConf *cf)
@@ -319,7 +427,7 @@ bool make_conf(const hdc_sweep_spec *sp, int64_t D, SweepConf *cf)
 }
 
 struct SweepLayout {
-    size_t planes, sums, norms, total;
+    size_t planes, sums, norms, total;   // tensor-core route: digit rows, sums of squares
 };
 
 SweepLayout sweep_layout(int D, int C, const SweepConf &cf)
@@ -328,6 +436,15 @@ SweepLayout sweep_layout(int D, int C, const SweepConf &cf)
     size_t off = 0;
     const int W = words_for(D);
     const size_t ncfg = (size_t)cf.nb * cf.ns;
+    SweepRows rw;
+    int rows;
+    if (sweep_rows(cf, C, W, &rw, &rows)) {
+        L.planes = off; off = align_up(off + (size_t)rows * hamming_packed_ldcs(W), kAlign);
+        L.sums = off;   off = align_up(off + ncfg * C * 8, kAlign);
+        L.norms = off;
+        L.total = off;
+        return L;
+    }
     L.planes = off; off = align_up(off + (size_t)cf.total_planes * C * W * 4, kAlign);
     L.sums = off;   off = align_up(off + ncfg * C * 8, kAlign);
     L.norms = off;  off = align_up(off + ncfg * C * 8, kAlign);
@@ -371,6 +488,38 @@ extern "C" hdc_status hdc_sweep_eval(const uint32_t *H, const int32_t *y, int64_
     cudaStream_t st = (cudaStream_t)stream;
     char *w = (char *)ws;
     if (cudaMemsetAsync(correct, 0, ncfg * sizeof(int32_t), st) != cudaSuccess) return HDC_ERR_CUDA;
+    SweepRows rw;
+    int rows;
+    if (sweep_rows(cf, C, W, &rw, &rows)) {
+        const int ld = hamming_packed_ldcs(W);
+        uint8_t *vals = (uint8_t *)(w + L.planes);
+        long long *sumsq = (long long *)(w + L.sums);
+        if (cudaMemsetAsync(sumsq, 0, ncfg * C * sizeof(long long), st) != cudaSuccess) return HDC_ERR_CUDA;
+        sweep_digits_kernel<<<dim3((unsigned)C, (unsigned)((ld + SPD - 1) / SPD)), 256, 0, st>>>(acc, D, C, ld, cf, rw,
+                                                                                                 vals, sumsq);
+        if (cudaGetLastError() != cudaSuccess) return HDC_ERR_CUDA;
+        if (N == 0) return HDC_OK;
+        PackedSweep a = {};
+        a.H = H;
+        a.y = y;
+        a.N = N;
+        a.W = W;
+        a.C = C;
+        a.sumsq = sumsq;
+        a.correct = correct;
+        a.labels = labels;
+        for (int f = 0; f < rw.n;) {   // passes of whole configurations, at most 256 class rows each
+            a.ncfg = 0;
+            a.vals = vals + (size_t)rw.row[f] * ld;
+            for (int n = 0; f < rw.n && n + C * rw.digits[f] <= 256; f++) {
+                n += C * rw.digits[f];
+                a.digits[a.ncfg] = cf.bits[rw.jb[f]] == 1 ? 0 : (uint8_t)rw.digits[f];
+                a.out[a.ncfg++] = (uint8_t)(rw.jb[f] * cf.ns + rw.entry[f]);
+            }
+            if (launch_packed_sweep(a, st) != cudaSuccess) return HDC_ERR_CUDA;
+        }
+        return HDC_OK;
+    }
     sweep_prep_kernel<<<C, 256, 0, st>>>(acc, D, C, W, cf, (uint32_t *)(w + L.planes), (long long *)(w + L.sums),
                                          (double *)(w + L.norms));
     if (cudaGetLastError() != cudaSuccess) return HDC_ERR_CUDA;

@@ -60,15 +60,15 @@ bool make_cls_map(CUtensorMap *m, const uint32_t *planes, int W, int C)
     return r == CUDA_SUCCESS;
 }
 
-// Map over the E4M3 +-1 class bytes (Cp rows x ldcs bytes): box = one
-// 128-byte K atom x Cp rows, 128-byte swizzle (the MMA operand layout).
-bool make_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int Cp)
+// Map over E4M3 class bytes (rows x ldcs bytes): box = one 128-byte K atom x
+// `box_rows` rows (zeros past `rows`), 128-byte swizzle (the MMA operand layout).
+bool make_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int rows, int box_rows)
 {
     auto fn = encode_fn();
     if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)ldcs, (cuuint64_t)Cp};
+    cuuint64_t dims[2] = {(cuuint64_t)ldcs, (cuuint64_t)rows};
     cuuint64_t strides[1] = {(cuuint64_t)ldcs};
-    cuuint32_t box[2] = {128, (cuuint32_t)Cp};
+    cuuint32_t box[2] = {128, (cuuint32_t)box_rows};
     cuuint32_t estr[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<uint8_t *>(signs), dims, strides, box, estr,
               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -86,9 +86,9 @@ int sm_count()
 }  // namespace
 
 // The class-byte map for the other tensor-core translation units.
-bool make_class_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int Cp)
+bool make_class_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int rows, int box)
 {
-    return make_sign_map(m, signs, ldcs, Cp);
+    return make_sign_map(m, signs, ldcs, rows, box);
 }
 
 bool make_packed_map(CUtensorMap *m, const uint32_t *Q, int W, int64_t N)
@@ -215,7 +215,7 @@ cudaError_t launch_tc_encode(const TcArgs &a, cudaStream_t st)
         // (F 617, D 2,048, 26 classes: 1.22 vs 1.59 ms per 2^20 queries)
         CUtensorMap mb2, ms;
         const int Cp = (a.C + 15) / 16 * 16;
-        if (!make_map(&mb2, a.Bq, a.enc, a.F, a.ldb, a.Dk, tc::HBN) || !make_sign_map(&ms, a.cls_sign, a.ldcs, Cp))
+        if (!make_map(&mb2, a.Bq, a.enc, a.F, a.ldb, a.Dk, tc::HBN) || !make_sign_map(&ms, a.cls_sign, a.ldcs, Cp, Cp))
             return cudaErrorInvalidValue;
         tc::HParams h;
         h.N = a.N;

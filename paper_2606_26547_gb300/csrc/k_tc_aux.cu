@@ -7,9 +7,10 @@
 
 namespace hdc {
 
-// Tensor map of E4M3 class bytes (Cp rows of ldcs bytes, boxes of 128 bytes x
-// Cp rows, 128-byte swizzle), defined with the other map builders.
-bool make_class_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int Cp);
+// Tensor map of E4M3 class bytes (`rows` rows of ldcs bytes, boxes of 128 bytes
+// x `box` rows, 128-byte swizzle, zeros past the rows), defined with the other
+// map builders.
+bool make_class_sign_map(CUtensorMap *m, const uint8_t *signs, int ldcs, int rows, int box);
 // Tensor map of packed rows (N rows of W words): boxes of 32 words x 128 rows,
 // 128-byte swizzle, zeros past W and N.
 bool make_packed_map(CUtensorMap *m, const uint32_t *Q, int W, int64_t N);
@@ -85,6 +86,44 @@ HpPlan hp_plan(int64_t N, int mt, int chunks, int sms, int tile_cost)
     pl.cost = waves * ((chunks + pl.S - 1) / pl.S) * tile_cost;
     return pl;
 }
+// Chooses the form of a task whose sizes and epilogue `p` holds, and launches
+// it: mq the packed rows, mc the class bytes (PRE).
+template <bool PRE, int FIN>
+cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensorMap &mc, cudaStream_t st)
+{
+    const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
+    HpPlan pl = hp_plan(p.N, 1, chunks, sms, 3);
+    if (p.R <= 128) {
+        const HpPlan p2 = hp_plan(p.N, 2, chunks, sms, 5);
+        if (p2.cost < pl.cost) pl = p2;
+    }
+    p.S = pl.S;
+    // shared memory: the query ring, the class atoms, barriers; at least 120 KB
+    // so that no second CTA shares the SM and waits for its TMEM columns
+    const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::hp_tail(pl.mt), atom = (size_t)p.R * 128;
+    size_t nbs = (227 * 1024 - fixed) / atom;
+    if (nbs > (size_t)tc::HP_NBS_MAX) nbs = tc::HP_NBS_MAX;
+    p.nbs = (int)nbs;
+    size_t smem = fixed + (PRE ? nbs * atom : tc::hp_nab(pl.mt, false) * atom + (size_t)((p.W + 3) & ~3) * 4);
+    if (smem < 120 * 1024) smem = 120 * 1024;
+    auto k = pl.mt == 2 ? tc::tc_hamming_packed_kernel<2, PRE, FIN> : tc::tc_hamming_packed_kernel<1, PRE, FIN>;
+    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    const int64_t ctas = pl.units * pl.S;
+    cudaLaunchConfig_t lc = {};
+    lc.gridDim = dim3((unsigned)(pl.S > 1 || ctas < sms ? ctas : sms));
+    lc.blockDim = dim3(tc::HP_THREADS);
+    lc.dynamicSmemBytes = smem;
+    lc.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = (unsigned)pl.S;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    lc.attrs = at;
+    lc.numAttrs = pl.S > 1 ? 1 : 0;
+    return cudaLaunchKernelEx(&lc, k, p, mq, mc);
+}
 }  // namespace
 
 // Form of a call.  Two 128-row tiles a unit halve the class bytes streamed per
@@ -114,9 +153,9 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
                                                                         reinterpret_cast<uint32_t *>(signs));
         const cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
-        if (!make_class_sign_map(&mc, signs, ldcs, R)) return cudaErrorInvalidValue;
+        if (!make_class_sign_map(&mc, signs, ldcs, C, R)) return cudaErrorInvalidValue;
     }
-    tc::HPParams p;
+    tc::HPParams p = {};
     p.cls = cls;
     p.N = N;
     p.W = W;
@@ -131,39 +170,59 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
     p.kept = end > s0 ? (int)((end - s0 + stride - 1) / stride) : 0;
     p.labels = labels;
     p.dists = dists;
-    const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
-    HpPlan pl = hp_plan(N, 1, chunks, sms, 3);
-    if (R <= 128) {
-        const HpPlan p2 = hp_plan(N, 2, chunks, sms, 5);
-        if (p2.cost < pl.cost) pl = p2;
+    return signs ? launch_packed<true, tc::HP_HAMMING>(p, mq, mc, st) : launch_packed<false, tc::HP_HAMMING>(p, mq, mc, st);
+}
+
+cudaError_t launch_packed_cosine(const uint32_t *Q, int64_t N, int W, const uint8_t *vals, int C, int P,
+                                 const double *cnorm, int32_t *labels, double *scores, cudaStream_t st)
+{
+    if (N <= 0) return cudaSuccess;
+    const int rows = C * P, R = (rows + 15) / 16 * 16, ld = hamming_packed_ldcs(W);
+    if (!hamming_packed_ok(rows, W) || P < 1 || P > 2 || N > 0x7fffffffLL - 2 * tc::BM) return cudaErrorNotSupported;
+    CUtensorMap mq, mc;
+    if (!make_packed_map(&mq, Q, W, N) || !make_class_sign_map(&mc, vals, ld, rows, R)) return cudaErrorInvalidValue;
+    tc::HPParams p = {};
+    p.N = N;
+    p.W = W;
+    p.C = C;
+    p.R = R;
+    p.nt = (W + 7) / 8;
+    p.P = P;
+    p.cnorm = cnorm;
+    p.labels = labels;
+    p.scores = scores;
+    return launch_packed<true, tc::HP_COSINE>(p, mq, mc, st);
+}
+
+cudaError_t launch_packed_sweep(const PackedSweep &a, cudaStream_t st)
+{
+    if (a.N <= 0 || a.ncfg <= 0) return cudaSuccess;
+    tc::HPParams p = {};
+    int rows = 0;
+    for (int i = 0; i < a.ncfg; i++) {
+        p.cfg_p[i] = a.digits[i];
+        p.cfg_k[i] = a.out[i];
+        p.cfg_col[i] = (uint16_t)rows;
+        rows += a.C * (a.digits[i] ? a.digits[i] : 1);
     }
-    p.S = pl.S;
-    // shared memory: the query ring, the class atoms, barriers; at least 120 KB
-    // so that no second CTA shares the SM and waits for its TMEM columns
-    const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::hp_tail(pl.mt), atom = (size_t)R * 128;
-    size_t nbs = (227 * 1024 - fixed) / atom;
-    if (nbs > (size_t)tc::HP_NBS_MAX) nbs = tc::HP_NBS_MAX;
-    p.nbs = (int)nbs;
-    size_t smem = fixed + (signs ? nbs * atom : tc::hp_nab(pl.mt, false) * atom + (size_t)((W + 3) & ~3) * 4);
-    if (smem < 120 * 1024) smem = 120 * 1024;
-    auto k = pl.mt == 2 ? (signs ? tc::tc_hamming_packed_kernel<2, true> : tc::tc_hamming_packed_kernel<2, false>)
-                        : (signs ? tc::tc_hamming_packed_kernel<1, true> : tc::tc_hamming_packed_kernel<1, false>);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    const int64_t ctas = pl.units * pl.S;
-    cudaLaunchConfig_t lc = {};
-    lc.gridDim = dim3((unsigned)(pl.S > 1 || ctas < sms ? ctas : sms));
-    lc.blockDim = dim3(tc::HP_THREADS);
-    lc.dynamicSmemBytes = smem;
-    lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)pl.S;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
-    lc.attrs = at;
-    lc.numAttrs = pl.S > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&lc, k, p, mq, mc);
+    if (a.ncfg > tc::HP_MAXCFG || !hamming_packed_ok(rows, a.W) || a.N > 0x7fffffffLL - 2 * tc::BM)
+        return cudaErrorNotSupported;
+    const int R = (rows + 15) / 16 * 16;
+    CUtensorMap mq, mc;
+    if (!make_packed_map(&mq, a.H, a.W, a.N) ||
+        !make_class_sign_map(&mc, a.vals, hamming_packed_ldcs(a.W), rows, R))
+        return cudaErrorInvalidValue;
+    p.N = a.N;
+    p.W = a.W;
+    p.C = a.C;
+    p.R = R;
+    p.nt = (a.W + 7) / 8;
+    p.ncfg = a.ncfg;
+    p.sumsq = a.sumsq;
+    p.y = a.y;
+    p.correct = a.correct;
+    p.labels = a.labels;
+    return launch_packed<true, tc::HP_SWEEP>(p, mq, mc, st);
 }
 
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st)

@@ -1,6 +1,15 @@
-// Packed +-1 rows against small-integer class rows on the tensor cores: the
-// Hamming arg-min of packed binary hypervectors (Sec. 4.1 Hamming distance
-// and arg-min primitives) for up to 256 classes.
+// Packed +-1 rows against small-integer class rows on the tensor cores (up to
+// 256 class rows).  What the dot products are for (FIN):
+//   HP_HAMMING  the Hamming arg-min of packed binary hypervectors (Sec. 4.1
+//               Hamming distance and arg-min primitives);
+//   HP_COSINE   the cosine arg-max against b-bit class hypervectors (Sec. 4.2
+//               Algorithmic Choice);
+//   HP_SWEEP    the arg-max of every (class width, perforation) configuration
+//               of a trained model, its correct predictions counted.
+// A b-bit class value is P signed base-16 digits (1 for up to 4 bits, 2 for 8,
+// 8 for 32), each a class row of its own that E4M3 holds exactly; the digits'
+// dot products, exact in FP32 (at most 8 * 131,072), are put together as
+// integers.
 //
 // For +-1 vectors over the kept dims K, Hamming(q, c) = (|K| - q.c) / 2, and
 // q.c is an exact integer in FP32.  The packed words are expanded to E4M3
@@ -61,6 +70,8 @@ constexpr int HP_QB = 3;                       // query chunks in the ring
 constexpr int HP_CHUNK = 4;                    // 256-dim tiles per query chunk (128 bytes of a row)
 constexpr int HP_NBS_MAX = 16;                 // most class-atom slots
 constexpr int HP_SMAX = 8;                     // most CTAs a unit's dims are split over
+constexpr int HP_HAMMING = 0, HP_COSINE = 1, HP_SWEEP = 2;
+constexpr int HP_MAXCFG = HDC_SWEEP_MAX_STRIDES * HDC_SWEEP_MAX_BITS;
 constexpr uint32_t HP_ACOL = 256;              // first TMEM column of the query buffers
 constexpr int HP_NAB_MAX = 8;                  // query-atom buffers: 4, or 8 with MT = 1 and PRE
 __host__ __device__ constexpr int hp_nab(int mt, bool pre) { return mt == 1 && pre ? 8 : 4; }
@@ -81,6 +92,20 @@ struct HPParams {
     int64_t D, s0, e0, stride;   // dims of the rows; kept dims s0 + k*stride < e0 (stride 1, [0, D) if none)
     int kept;                // |K|
     int32_t *labels, *dists;
+    // HP_COSINE: digits of a class value, class norms, optional scores (N x C)
+    int P;
+    const double *cnorm;
+    double *scores;
+    // HP_SWEEP: ncfg configurations of C classes; configuration i owns the
+    // class rows [cfg_col, cfg_col + C * cfg_p), class by class, its digits
+    // side by side (cfg_p 0: one sign row, Hamming), and writes output entry
+    // cfg_k; sumsq[cfg_k * C + c]: sum of the squared class values it keeps
+    int ncfg;
+    uint8_t cfg_p[HP_MAXCFG], cfg_k[HP_MAXCFG];
+    uint16_t cfg_col[HP_MAXCFG];
+    const long long *sumsq;
+    const int32_t *y;
+    int32_t *correct;
 };
 
 // Four dims j, j + 8, j + 16, j + 24 of a packed word as E4M3 +-1 bytes.
@@ -136,6 +161,29 @@ __device__ __forceinline__ void hp_expand_row(uint8_t *atom, int r, int p0, cons
     }
 }
 
+// Eight 32-bit TMEM columns of this thread's lane.
+__device__ __forceinline__ void hp_tmem_ld8(uint32_t taddr, uint32_t (&r)[8])
+{
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+                 : "r"(taddr));
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7])
+                 :
+                 : "memory");
+}
+
+// Value of P digit dot products (exact integers): the digits' weights are the
+// powers of 16.
+template <int P>
+__device__ __forceinline__ long long hp_digits(const uint32_t *v)
+{
+    long long d = 0;
+#pragma unroll
+    for (int q = P - 1; q >= 0; q--) d = d * 16 + (long long)(int)__uint_as_float(v[q]);
+    return d;
+}
+
 __device__ __forceinline__ void hp_cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -151,7 +199,12 @@ __device__ __forceinline__ float hp_ld_cluster(uint32_t a, uint32_t rank)
     return v;
 }
 
-template <int MT, bool PRE>
+template <int V>
+struct HpInt {
+    static constexpr int value = V;
+};
+
+template <int MT, bool PRE, int FIN = HP_HAMMING>
 __global__ void __launch_bounds__(HP_THREADS, 1)
     tc_hamming_packed_kernel(const HPParams p, const __grid_constant__ CUtensorMap tmQ,
                              const __grid_constant__ CUtensorMap tmC)
@@ -212,6 +265,14 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    double *s_norm = reinterpret_cast<double *>(s_out);   // class norms (cosine, sweep: no distances are staged)
+    if (FIN == HP_COSINE)
+        for (int i = tid; i < p.C; i += HP_THREADS) s_norm[i] = p.cnorm[i];
+    if (FIN == HP_SWEEP)
+        for (int i = tid; i < p.ncfg * p.C; i += HP_THREADS) {
+            const int f = i / p.C;
+            s_norm[i] = p.cfg_p[f] ? sqrt((double)p.sumsq[(int64_t)p.cfg_k[f] * p.C + i % p.C]) : 1.0;
+        }
     if (!PRE)
         for (int w = tid; w < p.W; w += HP_THREADS) smask[w] = hp_word_mask(w, p.D, p.s0, p.e0, p.stride);
     if (warp == 0) {
@@ -266,6 +327,65 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             }
         }
         if (lane < nrow) p.labels[row0 + lane] = best;
+    };
+
+    // Cosine arg-max of this lane's row from its C * P digit dot products,
+    // read eight columns at a time by cols8(col, v).  Scores and their order
+    // are those of the general kernel: dot / norm in FP64, lowest class first.
+    auto arg_max = [&](int64_t row, bool valid, int col, const double *norm, double *scores, auto digits, auto cols8) {
+        constexpr int P = decltype(digits)::value, CPL = 8 / P;   // classes a load
+        int best = 0;
+        double bs = 0.0;
+        for (int c0 = 0; c0 < p.C; c0 += CPL) {
+            uint32_t v[8];
+            cols8(col + c0 * P, v);
+#pragma unroll
+            for (int i = 0; i < CPL; i++) {
+                const int c = c0 + i;
+                if (c < p.C) {
+                    const double n = norm[c];
+                    const double sc = n == 0.0 ? 0.0 : (double)hp_digits<P>(v + i * P) / n;
+                    if (scores && valid) scores[row * p.C + c] = sc;
+                    if (c == 0 || sc > bs) { bs = sc; best = c; }
+                }
+            }
+        }
+        return best;
+    };
+    auto finish_scores = [&](int64_t row0, auto cols8) {
+        const int64_t row = row0 + lane;
+        const bool valid = row < p.N;
+        if (FIN == HP_COSINE) {
+            const int best = p.P == 1 ? arg_max(row, valid, 0, s_norm, p.scores, HpInt<1>(), cols8)
+                                      : arg_max(row, valid, 0, s_norm, p.scores, HpInt<2>(), cols8);
+            if (valid) p.labels[row] = best;
+            return;
+        }
+        const int yv = valid ? p.y[row] : -1;
+        for (int f = 0; f < p.ncfg; f++) {
+            const double *norm = s_norm + f * p.C;
+            const int col = p.cfg_col[f];
+            int best = 0;
+            if (p.cfg_p[f] == 0) {   // signs: the largest dot product is the smallest distance
+                float bd = -3.0e38f;
+                for (int c0 = 0; c0 < p.C; c0 += 8) {
+                    uint32_t v[8];
+                    cols8(col + c0, v);
+#pragma unroll
+                    for (int i = 0; i < 8; i++)
+                        if (c0 + i < p.C && __uint_as_float(v[i]) > bd) { bd = __uint_as_float(v[i]); best = c0 + i; }
+                }
+            } else if (p.cfg_p[f] == 1) {
+                best = arg_max(row, valid, col, norm, nullptr, HpInt<1>(), cols8);
+            } else if (p.cfg_p[f] == 2) {
+                best = arg_max(row, valid, col, norm, nullptr, HpInt<2>(), cols8);
+            } else {
+                best = arg_max(row, valid, col, norm, nullptr, HpInt<8>(), cols8);
+            }
+            if (valid && p.labels) p.labels[(int64_t)p.cfg_k[f] * p.N + row] = best;
+            const unsigned hit = __ballot_sync(0xffffffffu, valid && best == yv);
+            if (lane == 0 && hit) atomicAdd(p.correct + p.cfg_k[f], __popc(hit));
+        }
     };
 
     if (warp == HP_ISSUER) {
@@ -441,7 +561,10 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             if (!__all_sync(0xffffffffu, okd)) break;
             tc_fence_after();
             const uint32_t dcol = tmem + tlane + (uint32_t)((d2 * MT + (e >> 2)) * RS);
-            if (S == 1) {
+            if (S == 1 && FIN != HP_HAMMING) {
+                finish_scores(u * UROWS + e * 32,
+                              [&](int col, uint32_t(&v)[8]) { hp_tmem_ld8(dcol + (uint32_t)col, v); });
+            } else if (S == 1) {
                 finish(u * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) { tmem_ld32(dcol + (uint32_t)(j * 32), v); });
             } else {   // this rank's partial sums, [column][row of the unit], over the rings (all consumed)
                 float *dump = reinterpret_cast<float *>(smem) + e * 32 + lane;
@@ -466,15 +589,22 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         const int e = warp - HP_EPI0;
         if (e >= 0 && e < 4 * MT && e % S == rank && u0 < units) {
             const uint32_t base = su32(smem) + (uint32_t)(e * 32 + lane) * 4u;
-            finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) {
+            auto total = [&](int col) {
+                float t = 0.f;
+                if (col < p.R)
+                    for (int k = 0; k < S; k++) t += hp_ld_cluster(base + (uint32_t)(col * UROWS) * 4u, (uint32_t)k);
+                return __float_as_uint(t);
+            };
+            if (FIN == HP_HAMMING)
+                finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) {
 #pragma unroll
-                for (int i = 0; i < 32; i++) {
-                    float s = 0.f;
-                    if (j * 32 + i < p.R)
-                        for (int k = 0; k < S; k++) s += hp_ld_cluster(base + (uint32_t)((j * 32 + i) * UROWS) * 4u, (uint32_t)k);
-                    v[i] = __float_as_uint(s);
-                }
-            });
+                    for (int i = 0; i < 32; i++) v[i] = total(j * 32 + i);
+                });
+            else
+                finish_scores(u0 * UROWS + e * 32, [&](int col, uint32_t(&v)[8]) {
+#pragma unroll
+                    for (int i = 0; i < 8; i++) v[i] = total(col + i);
+                });
         }
         __syncwarp();
         hp_cluster_sync();
