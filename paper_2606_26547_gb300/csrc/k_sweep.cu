@@ -278,12 +278,12 @@ struct SweepRows {
 
 __device__ __forceinline__ uint32_t entry_mask(const SweepConf &cf, int i, int w);
 
-// A block takes one class and 1,024 dims (a thread four dims of one word),
-// after scanning all of the class's accumulators for its largest magnitude;
-// the squares of the kept values are added into sumsq (zeroed by the caller).
-// One block a class for everything took most of the time of a short sweep.
-constexpr int SPD = 1024;
-__global__ void __launch_bounds__(256) sweep_digits_kernel(const int32_t *__restrict__ acc, int D, int C, int ld,
+// A block takes one class, 1,024 dims (a thread four dims of one word) and one
+// width, after scanning all of the class's accumulators for its largest
+// magnitude; the squares of the kept values are added into sumsq (zeroed by the
+// caller).  64-bit divisions and shuffles only where the values need them.
+constexpr int SPD = 1024, SPT = SPD / 4;
+__global__ void __launch_bounds__(SPT) sweep_digits_kernel(const int32_t *__restrict__ acc, int D, int C, int ld,
                                                            const __grid_constant__ SweepConf cf,
                                                            const __grid_constant__ SweepRows rw,
                                                            uint8_t *__restrict__ vals, long long *__restrict__ sumsq)
@@ -295,35 +295,52 @@ __global__ void __launch_bounds__(256) sweep_digits_kernel(const int32_t *__rest
     if (tid == 0) s_max = 0;
     if (tid < MAXB * MAXS) s_sq[tid] = 0;
     __syncthreads();
-    unsigned m = 0;   // |acc| < 2^31; -2^31 itself has magnitude 2^31 in 32 bits unsigned
-#pragma unroll 8
-    for (int d = tid; d < D; d += 256) {
+    unsigned m = 0;   // magnitudes up to 2^31
+#pragma unroll 16
+    for (int d = tid; d < D; d += SPT) {
         const int v = __ldg(a + d);
         m = max(m, v < 0 ? 0u - (unsigned)v : (unsigned)v);
     }
     m = __reduce_max_sync(0xffffffffu, m);
     if ((tid & 31) == 0) atomicMax(&s_max, m);
     __syncthreads();
-    const long long M = s_max;
+    const unsigned M = s_max;
     const int w = blockIdx.y * (SPD / 32) + (tid >> 3), j = tid & 7;   // dims 32w + j + 8k, k = 0..3
-    long long x[4];
+    int x[4];
 #pragma unroll
     for (int k = 0; k < 4; k++) {
         const int d = w * 32 + j + 8 * k;
-        x[k] = d < D ? (long long)__ldg(a + d) : 0;
+        x[k] = d < D ? __ldg(a + d) : 0;
     }
-    for (int jb = 0; jb < cf.nb; jb++) {
-        long long v[4];
+    {
+        const int jb = blockIdx.z, b = cf.bits[jb];
+        int v[4];   // class values: every width fits 32 bits
+        const unsigned Q = b > 1 ? (1u << (b - 1)) - 1u : 0u;
 #pragma unroll
-        for (int k = 0; k < 4; k++) v[k] = w * 32 + j + 8 * k < D ? class_value(x[k], cf.bits[jb], M) : 0;
+        for (int k = 0; k < 4; k++) {
+            if (w * 32 + j + 8 * k >= D) v[k] = 0;
+            else if (b > 1 && M > 0 && M < (1u << 23)) {   // 2 |acc| Q + M < 2^32: a 32-bit division
+                const unsigned mag = x[k] < 0 ? 0u - (unsigned)x[k] : (unsigned)x[k];
+                const int r = (int)((2u * mag * Q + M) / (2u * M));
+                v[k] = x[k] < 0 ? -r : r;
+            } else
+                v[k] = (int)class_value(x[k], b, M);
+        }
         for (int f = 0; f < rw.n; f++) {
             if (rw.jb[f] != jb) continue;
             const uint32_t em = entry_mask(cf, rw.entry[f], w) >> j;
-            long long r[4], sq = 0;
+            long long r[4];
 #pragma unroll
-            for (int k = 0; k < 4; k++) {
-                r[k] = (em >> (8 * k)) & 1u ? v[k] : 0;
-                sq += r[k] * r[k];
+            for (int k = 0; k < 4; k++) r[k] = (em >> (8 * k)) & 1u ? v[k] : 0;
+            if (b != 0) {   // at most 32 lanes x 4 x 127^2
+                const unsigned sq = __reduce_add_sync(0xffffffffu, (unsigned)((int)r[0] * (int)r[0] + (int)r[1] * (int)r[1] +
+                                                                             (int)r[2] * (int)r[2] + (int)r[3] * (int)r[3]));
+                if ((tid & 31) == 0 && sq) atomicAdd(&s_sq[f], (unsigned long long)sq);
+            } else {
+                long long sq = r[0] * r[0] + r[1] * r[1] + r[2] * r[2] + r[3] * r[3];
+#pragma unroll
+                for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
+                if ((tid & 31) == 0 && sq) atomicAdd(&s_sq[f], (unsigned long long)sq);
             }
             if (w * 32 < ld) {
                 uint32_t *o = reinterpret_cast<uint32_t *>(vals + (int64_t)(rw.row[f] + c * rw.digits[f]) * ld + w * 32) + j;
@@ -338,13 +355,10 @@ __global__ void __launch_bounds__(256) sweep_digits_kernel(const int32_t *__rest
                     o[(int64_t)q * (ld / 4)] = to_e4m3x4(g[0], g[1], g[2], g[3]);
                 }
             }
-#pragma unroll
-            for (int o = 16; o; o >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, o);
-            if ((tid & 31) == 0 && sq) atomicAdd(&s_sq[f], (unsigned long long)sq);
         }
     }
     __syncthreads();
-    if (tid < rw.n && s_sq[tid])
+    if (tid < rw.n && s_sq[tid])   // this width's entries; the others stay zero here
         atomicAdd((unsigned long long *)sumsq + (int64_t)(rw.jb[tid] * cf.ns + rw.entry[tid]) * C + c, s_sq[tid]);
 }
 
@@ -495,7 +509,7 @@ extern "C" hdc_status hdc_sweep_eval(const uint32_t *H, const int32_t *y, int64_
         uint8_t *vals = (uint8_t *)(w + L.planes);
         long long *sumsq = (long long *)(w + L.sums);
         if (cudaMemsetAsync(sumsq, 0, ncfg * C * sizeof(long long), st) != cudaSuccess) return HDC_ERR_CUDA;
-        sweep_digits_kernel<<<dim3((unsigned)C, (unsigned)((ld + SPD - 1) / SPD)), 256, 0, st>>>(acc, D, C, ld, cf, rw,
+        sweep_digits_kernel<<<dim3((unsigned)C, (unsigned)((ld + SPD - 1) / SPD), (unsigned)cf.nb), SPT, 0, st>>>(acc, D, C, ld, cf, rw,
                                                                                                  vals, sumsq);
         if (cudaGetLastError() != cudaSuccess) return HDC_ERR_CUDA;
         if (N == 0) return HDC_OK;

@@ -184,6 +184,28 @@ __device__ __forceinline__ long long hp_digits(const uint32_t *v)
     return d;
 }
 
+// The same rounded once to FP32: exact for P <= 2 (below 2^24).  Eight digits
+// may cancel, so they are put together as integers first.
+template <int P>
+__device__ __forceinline__ float hp_digits_f(const uint32_t *v)
+{
+    if (P == 1) return __uint_as_float(v[0]);
+    if (P == 2) return fmaf(__uint_as_float(v[1]), 16.f, __uint_as_float(v[0]));
+    return (float)hp_digits<P>(v);
+}
+
+// a / b correctly rounded from y = 1 / b correctly rounded (0 for b = 0, which
+// gives 0): P. Markstein, "Computation of elementary functions on the IBM RISC
+// System/6000 processor", IBM J. Res. Dev. 34(1), 1990: one step makes the
+// quotient faithful, the next one correct.  Integers a and norms b: no
+// overflow, no subnormals.
+__device__ __forceinline__ double hp_div(double a, double b, double y)
+{
+    double q = a * y;
+    q = fma(fma(-q, b, a), y, q);
+    return fma(fma(-q, b, a), y, q);
+}
+
 __device__ __forceinline__ void hp_cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
@@ -194,8 +216,7 @@ __device__ __forceinline__ float hp_ld_cluster(uint32_t a, uint32_t rank)
     float v;
     asm volatile("{\n\t.reg .b32 r;\n\tmapa.shared::cluster.u32 r, %1, %2;\n\tld.shared::cluster.f32 %0, [r];\n\t}"
                  : "=f"(v)
-                 : "r"(a), "r"(rank)
-                 : "memory");
+                 : "r"(a), "r"(rank));
     return v;
 }
 
@@ -265,13 +286,18 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    double *s_norm = reinterpret_cast<double *>(s_out);   // class norms (cosine, sweep: no distances are staged)
-    if (FIN == HP_COSINE)
-        for (int i = tid; i < p.C; i += HP_THREADS) s_norm[i] = p.cnorm[i];
-    if (FIN == HP_SWEEP)
-        for (int i = tid; i < p.ncfg * p.C; i += HP_THREADS) {
-            const int f = i / p.C;
-            s_norm[i] = p.cfg_p[f] ? sqrt((double)p.sumsq[(int64_t)p.cfg_k[f] * p.C + i % p.C]) : 1.0;
+    // class norms and their reciprocals, 0 for a zero norm (cosine, sweep: no
+    // distances are staged there)
+    double *s_norm = reinterpret_cast<double *>(s_out), *s_rinv = s_norm + HP_CMAX;
+    float *s_rinvf = reinterpret_cast<float *>(s_rinv + HP_CMAX);   // (narrowing takes the FP64 pipe: once here)
+    if (FIN != HP_HAMMING)
+        for (int i = tid; i < (FIN == HP_SWEEP ? p.ncfg : 1) * p.C; i += HP_THREADS) {
+            const int f = FIN == HP_SWEEP ? i / p.C : 0;
+            const double n = FIN == HP_COSINE ? p.cnorm[i] : sqrt((double)p.sumsq[(int64_t)p.cfg_k[f] * p.C + i % p.C]);
+            s_norm[i] = n;
+            const double y = n == 0.0 ? 0.0 : 1.0 / n;
+            s_rinv[i] = y;
+            s_rinvf[i] = (float)y;
         }
     if (!PRE)
         for (int w = tid; w < p.W; w += HP_THREADS) smask[w] = hp_word_mask(w, p.D, p.s0, p.e0, p.stride);
@@ -330,23 +356,68 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     };
 
     // Cosine arg-max of this lane's row from its C * P digit dot products,
-    // read eight columns at a time by cols8(col, v).  Scores and their order
-    // are those of the general kernel: dot / norm in FP64, lowest class first.
-    auto arg_max = [&](int64_t row, bool valid, int col, const double *norm, double *scores, auto digits, auto cols8) {
+    // read eight columns at a time by cols8(col, v).  The score is dot / norm
+    // in FP64, lowest class first, as in the general kernel.  FP64 runs at a
+    // few operations per clock per SM here, so the arg-max alone is taken in
+    // FP32 (dot, 1 / norm and their product each rounded: within 2^-22 of the
+    // score) and only classes within 2^-20 of the largest are compared in FP64:
+    // a class below that cannot reach it.  With FP64 divisions for all, the
+    // sweep's epilogue took 75 of its 86 us.
+    auto arg_max = [&](int64_t row, bool valid, int col, int f0, double *scores, auto digits, auto cols8) {
         constexpr int P = decltype(digits)::value, CPL = 8 / P;   // classes a load
         int best = 0;
-        double bs = 0.0;
-        for (int c0 = 0; c0 < p.C; c0 += CPL) {
-            uint32_t v[8];
-            cols8(col + c0 * P, v);
+        if (scores) {
+            double bs = 0.0;
+            for (int c0 = 0; c0 < p.C; c0 += CPL) {
+                uint32_t v[8];
+                cols8(col + c0 * P, v);
 #pragma unroll
-            for (int i = 0; i < CPL; i++) {
-                const int c = c0 + i;
-                if (c < p.C) {
-                    const double n = norm[c];
-                    const double sc = n == 0.0 ? 0.0 : (double)hp_digits<P>(v + i * P) / n;
-                    if (scores && valid) scores[row * p.C + c] = sc;
-                    if (c == 0 || sc > bs) { bs = sc; best = c; }
+                for (int i = 0; i < CPL; i++) {
+                    const int c = c0 + i;
+                    if (c < p.C) {
+                        const double sc = hp_div((double)(int)hp_digits<P>(v + i * P), s_norm[f0 + c], s_rinv[f0 + c]);
+                        if (valid) scores[row * p.C + c] = sc;
+                        if (c == 0 || sc > bs) { bs = sc; best = c; }
+                    }
+                }
+            }
+            return best;
+        }
+        float top = -3.0e38f;
+        int near_top = 0;   // classes that may reach the largest score
+        for (int pass = 0; pass < 2; pass++) {
+            const float lim = top - fabsf(top) * 0x1p-20f;
+            for (int c0 = 0; c0 < p.C; c0 += CPL) {
+                uint32_t v[8];
+                cols8(col + c0 * P, v);
+#pragma unroll
+                for (int i = 0; i < CPL; i++) {
+                    const int c = c0 + i;
+                    if (c >= p.C) continue;
+                    const float sc = hp_digits_f<P>(v + i * P) * s_rinvf[f0 + c];
+                    if (pass == 0) {
+                        top = fmaxf(top, sc);
+                    } else if (sc >= lim) {
+                        if (near_top++ == 0) best = c;
+                    }
+                }
+            }
+        }
+        if (__any_sync(0xffffffffu, near_top > 1)) {   // a near tie in this warp: those rows again in FP64
+            const float lim = top - fabsf(top) * 0x1p-20f;
+            double bs = 0.0;
+            bool first = true;
+            for (int c0 = 0; c0 < p.C; c0 += CPL) {
+                uint32_t v[8];
+                cols8(col + c0 * P, v);
+#pragma unroll
+                for (int i = 0; i < CPL; i++) {
+                    const int c = c0 + i;
+                    if (c >= p.C) continue;
+                    const long long d = hp_digits<P>(v + i * P);
+                    if (hp_digits_f<P>(v + i * P) * s_rinvf[f0 + c] < lim) continue;
+                    const double n = s_norm[f0 + c], sc = n == 0.0 ? 0.0 : (double)d / n;
+                    if (first || sc > bs) { bs = sc; best = c; first = false; }
                 }
             }
         }
@@ -356,14 +427,13 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         const int64_t row = row0 + lane;
         const bool valid = row < p.N;
         if (FIN == HP_COSINE) {
-            const int best = p.P == 1 ? arg_max(row, valid, 0, s_norm, p.scores, HpInt<1>(), cols8)
-                                      : arg_max(row, valid, 0, s_norm, p.scores, HpInt<2>(), cols8);
+            const int best = p.P == 1 ? arg_max(row, valid, 0, 0, p.scores, HpInt<1>(), cols8)
+                                      : arg_max(row, valid, 0, 0, p.scores, HpInt<2>(), cols8);
             if (valid) p.labels[row] = best;
             return;
         }
         const int yv = valid ? p.y[row] : -1;
         for (int f = 0; f < p.ncfg; f++) {
-            const double *norm = s_norm + f * p.C;
             const int col = p.cfg_col[f];
             int best = 0;
             if (p.cfg_p[f] == 0) {   // signs: the largest dot product is the smallest distance
@@ -376,11 +446,11 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                         if (c0 + i < p.C && __uint_as_float(v[i]) > bd) { bd = __uint_as_float(v[i]); best = c0 + i; }
                 }
             } else if (p.cfg_p[f] == 1) {
-                best = arg_max(row, valid, col, norm, nullptr, HpInt<1>(), cols8);
+                best = arg_max(row, valid, col, f * p.C, nullptr, HpInt<1>(), cols8);
             } else if (p.cfg_p[f] == 2) {
-                best = arg_max(row, valid, col, norm, nullptr, HpInt<2>(), cols8);
+                best = arg_max(row, valid, col, f * p.C, nullptr, HpInt<2>(), cols8);
             } else {
-                best = arg_max(row, valid, col, norm, nullptr, HpInt<8>(), cols8);
+                best = arg_max(row, valid, col, f * p.C, nullptr, HpInt<8>(), cols8);
             }
             if (valid && p.labels) p.labels[(int64_t)p.cfg_k[f] * p.N + row] = best;
             const unsigned hit = __ballot_sync(0xffffffffu, valid && best == yv);
@@ -589,22 +659,30 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         const int e = warp - HP_EPI0;
         if (e >= 0 && e < 4 * MT && e % S == rank && u0 < units) {
             const uint32_t base = su32(smem) + (uint32_t)(e * 32 + lane) * 4u;
-            auto total = [&](int col) {
-                float t = 0.f;
-                if (col < p.R)
-                    for (int k = 0; k < S; k++) t += hp_ld_cluster(base + (uint32_t)(col * UROWS) * 4u, (uint32_t)k);
-                return __float_as_uint(t);
+            // the ranks' sums of this row, sixteen columns at a time, into this
+            // rank's own copy (no other rank reads these rows)
+            float *own = reinterpret_cast<float *>(smem) + e * 32 + lane;
+            for (int col = 0; col < p.R; col += 16) {   // R is a multiple of 16
+                float t[16];
+#pragma unroll
+                for (int i = 0; i < 16; i++) t[i] = 0.f;
+                for (int k = 0; k < S; k++)
+#pragma unroll
+                    for (int i = 0; i < 16; i++)
+                        t[i] += hp_ld_cluster(base + (uint32_t)((col + i) * UROWS) * 4u, (uint32_t)k);
+#pragma unroll
+                for (int i = 0; i < 16; i++) own[(col + i) * UROWS] = t[i];
+            }
+            auto sums = [&](int col, uint32_t *v, auto count) {
+#pragma unroll
+                for (int i = 0; i < decltype(count)::value; i++)
+                    v[i] = col + i < p.R ? __float_as_uint(own[(col + i) * UROWS]) : 0u;
             };
             if (FIN == HP_HAMMING)
-                finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4), [&](int j, uint32_t(&v)[32]) {
-#pragma unroll
-                    for (int i = 0; i < 32; i++) v[i] = total(j * 32 + i);
-                });
+                finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4),
+                       [&](int j, uint32_t(&v)[32]) { sums(j * 32, v, HpInt<32>()); });
             else
-                finish_scores(u0 * UROWS + e * 32, [&](int col, uint32_t(&v)[8]) {
-#pragma unroll
-                    for (int i = 0; i < 8; i++) v[i] = total(col + i);
-                });
+                finish_scores(u0 * UROWS + e * 32, [&](int col, uint32_t(&v)[8]) { sums(col, v, HpInt<8>()); });
         }
         __syncwarp();
         hp_cluster_sync();
