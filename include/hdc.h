@@ -145,7 +145,12 @@ typedef struct {
                                /* E4M3 +-1 bytes of the class hypervectors  */
                                /* (0 past Dk and for the pad classes up to  */
                                /* Cp = C rounded to 16) for the tensor-core */
-                               /* Hamming distances; NULL otherwise         */
+                               /* Hamming distances; 4- and 8-bit classes   */
+                               /* of binary queries, C * bits / 4 <= 256:   */
+                               /* E4M3 rows of their base-16 digits, bits/4 */
+                               /* a class (low digit first, byte 4j + k of  */
+                               /* a 32-dim word its dim j + 8k, 0 past Dk); */
+                               /* NULL otherwise                            */
     int32_t ldcs;              /* bytes per row of cls_sign                 */
     int32_t Fk;                /* kept features F' (= F without encoding    */
                                /* perforation); Bq rows hold these          */

@@ -88,6 +88,21 @@ inline bool tc_hamming_classes(int bits, int C, uint32_t flags)
 }
 inline int ldcs_for(int Dk) { return (Dk + 191) / 192 * 192 + 64; }
 
+// b-bit classes of binary queries keep their values as rows of E4M3 base-16
+// digits (b / 4 a class) for the tensor-core cosine, up to 256 rows.
+inline bool tc_cosine_classes(int bits, int C, int W, uint32_t flags)
+{
+    return bits > 1 && C > 0 && !(flags & HDC_FLAG_FLOAT_QUERY) && C <= 256 / (bits / 4) &&
+           hamming_packed_ok(C * (bits / 4), W);
+}
+// Bytes of the model's class rows for the tensor cores (0: none).
+inline size_t class_rows_bytes(int bits, int C, int Dk, uint32_t flags)
+{
+    const int W = words_for(Dk);
+    if (tc_cosine_classes(bits, C, W, flags)) return (size_t)C * (bits / 4) * hamming_packed_ldcs(W);
+    return tc_hamming_classes(bits, C, flags) ? (size_t)((C + 15) / 16 * 16) * ldcs_for(Dk) : 0;
+}
+
 ModelLayout model_layout(int F, int Dk, int C, int enc, int bits, uint32_t flags)
 {
     ModelLayout L;
@@ -101,7 +116,7 @@ ModelLayout model_layout(int F, int Dk, int C, int enc, int bits, uint32_t flags
     L.csum = off;   off = align_up(off + (size_t)C * 4, kAlign);
     L.cnorm = off;  off = align_up(off + (size_t)C * 8, kAlign);
     L.csign = off;
-    off = align_up(off + (tc_hamming_classes(bits, C, flags) ? (size_t)cpad_for(C) * ldcs_for(Dk) : 0), kAlign);
+    off = align_up(off + class_rows_bytes(bits, C, Dk, flags), kAlign);
     L.total = off;
     return L;
 }
@@ -283,10 +298,14 @@ hdc_status hdc_model_prepare(const float *Bt, int32_t F, int32_t D, const int32_
             s = cu(cudaMemsetAsync(b + L.planes, 0, L.csum - L.planes, st));
             if (s != HDC_OK) return s;
         }
+        if (tc_cosine_classes(bits, C, m.W, cfg->flags)) {
+            m.cls_sign = (const uint8_t *)(b + L.csign);
+            m.ldcs = hamming_packed_ldcs(m.W);
+        }
         s = cu(launch_class_prepare(acc, C, D, p, bits, (uint32_t *)(b + L.planes), m.W, (int32_t *)(b + L.csum),
                                     (double *)(b + L.cnorm),
                                     float_query(cfg->flags) ? (uint16_t *)(b + L.planes) : nullptr, lds_for(Dk),
-                                    st));
+                                    st, const_cast<uint8_t *>(m.cls_sign), m.ldcs));
         if (s != HDC_OK) return s;
         if (tc_hamming_classes(bits, C, cfg->flags)) {
             m.cls_sign = (const uint8_t *)(b + L.csign);
@@ -548,6 +567,11 @@ hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m, int32_t *
     if (classify_sign_bytes(m)) {   // 129..256 binary classes: the classes expanded once, then the tensor cores
         return cu(launch_hamming_packed(Hb, N, m->cls, m->C, m->W, m->Dk, 0, m->Dk, 1, labels, dists, st,
                                         (uint8_t *)ws + L.csign));
+    }
+    if (nb > 1 && m->cls_sign && m->ldcs == hamming_packed_ldcs(m->W) && m->C <= 256 / (nb / 4)) {
+        // b-bit classes on the tensor cores, where the model holds their digit rows
+        const cudaError_t e = launch_packed_cosine(Hb, N, m->W, m->cls_sign, m->C, nb / 4, m->cls_norm, labels, scores, st);
+        if (e != cudaErrorNotSupported) return cu(e);
     }
     return cu(launch_similarity(Hb, N, m->cls, m->C, m->W, nb, m->Dk, nullptr, m->cls_sum, m->cls_norm, labels,
                                 dists, scores, st));

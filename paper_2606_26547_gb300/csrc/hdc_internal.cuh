@@ -52,10 +52,12 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
                               cudaStream_t st, int64_t c0 = 0, int64_t cstep = 1);
 
 // Class preparation: planes [b][C][W] (or, with vals, the b-bit values as
-// BF16 rows of ldv elements, zero past Dk), sums and norms over the kept dims.
+// BF16 rows of ldv elements, zero past Dk), sums and norms over the kept dims;
+// with digits (b 4 or 8), also the values' b / 4 base-16 digit rows of ldd bytes
+// for the packed cosine kernel.
 cudaError_t launch_class_prepare(const int32_t *acc, int C, int D, const Perf &p, int b,
                                  uint32_t *planes, int W, int32_t *csum, double *cnorm,
-                                 uint16_t *vals, int ldv, cudaStream_t st);
+                                 uint16_t *vals, int ldv, cudaStream_t st, uint8_t *digits = nullptr, int ldd = 0);
 
 // Binary class planes (C x W words) -> E4M3 +-1 bytes (Cp x ldcs; 0 past Dk
 // and for rows C..Cp-1) for the tensor-core Hamming distances.

@@ -338,7 +338,8 @@ __global__ void __launch_bounds__(256) class_prepare_kernel(const int32_t *__res
                                                             int64_t stride, int64_t Dk, int b, int C,
                                                             uint32_t *__restrict__ planes, int W,
                                                             int32_t *__restrict__ csum, double *__restrict__ cnorm,
-                                                            uint16_t *__restrict__ vals, int ldv)
+                                                            uint16_t *__restrict__ vals, int ldv,
+                                                            uint8_t *__restrict__ digits, int ldd)
 {
     __shared__ long long s_max;
     __shared__ long long s_sum, s_sq;
@@ -361,7 +362,9 @@ __global__ void __launch_bounds__(256) class_prepare_kernel(const int32_t *__res
     const long long Q = (1ll << (b - 1)) - 1;
     long long lsum = 0, lsq = 0;
     // with vals: the row of ldv BF16 values (integers |v| <= 127: exact)
-    const int nwords = vals ? (ldv + 31) / 32 : W;
+    // with digits: the class's base-16 digit rows too (b / 4 of them, ldd
+    // bytes each, in the packed kernel's dim order, zero past Dk)
+    const int nwords = vals ? (ldv + 31) / 32 : digits ? ldd / 32 : W;
     for (int w = warp; w < nwords; w += nw) {
         int64_t k = (int64_t)w * 32 + lane;
         long long val = 0;
@@ -381,6 +384,13 @@ __global__ void __launch_bounds__(256) class_prepare_kernel(const int32_t *__res
         if (vals) {
             if (k < ldv) vals[(int64_t)c * ldv + k] = __bfloat16_as_ushort(__float2bfloat16_rn((float)val));
             continue;
+        }
+        if (digits) {
+            uint8_t *o = digits + (int64_t)c * (b / 4) * ldd + (int64_t)w * 32 + 4 * (lane & 7) + (lane >> 3);
+            const int lo = b == 8 ? (int)((val + 8) & 15) - 8 : (int)val;   // signed digits -8..7, then what is left
+            o[0] = (uint8_t)to_e4m3x4((float)lo, 0.f, 0.f, 0.f);
+            if (b == 8) o[ldd] = (uint8_t)to_e4m3x4((float)((int)(val - lo) / 16), 0.f, 0.f, 0.f);
+            if (w >= W) continue;   // the same for the whole warp
         }
         for (int j = 0; j < b; j++) {
             // b == 1: the single plane is the sign (set bit = element -1)
@@ -495,10 +505,12 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
 }
 
 cudaError_t launch_class_prepare(const int32_t *acc, int C, int D, const Perf &p, int b, uint32_t *planes, int W,
-                                 int32_t *csum, double *cnorm, uint16_t *vals, int ldv, cudaStream_t st)
+                                 int32_t *csum, double *cnorm, uint16_t *vals, int ldv, cudaStream_t st,
+                                 uint8_t *digits, int ldd)
 {
     if (C <= 0) return cudaSuccess;
-    class_prepare_kernel<<<C, 256, 0, st>>>(acc, D, p.s0, p.stride, p.Dk, b, C, planes, W, csum, cnorm, vals, ldv);
+    class_prepare_kernel<<<C, 256, 0, st>>>(acc, D, p.s0, p.stride, p.Dk, b, C, planes, W, csum, cnorm, vals, ldv, digits,
+                                            ldd);
     return cudaGetLastError();
 }
 
