@@ -164,8 +164,10 @@ WsLayout ws_layout(int64_t N, const hdc_model *m)
 hdc_status cu(cudaError_t e) { return e == cudaSuccess ? HDC_OK : HDC_ERR_CUDA; }
 
 // Quantise X into the workspace (BF16/FP8); returns the operand to encode.
+// The same launch zeroes the zero_n words at zero.
 hdc_status prepare_queries(const float *X, int64_t N, const hdc_model *m, char *ws, const WsLayout &L,
-                           const void **Xop, int64_t *ldx, const float **sx, cudaStream_t st)
+                           const void **Xop, int64_t *ldx, const float **sx, cudaStream_t st,
+                           uint32_t *zero = nullptr, int64_t zero_n = 0)
 {
     if (m->enc == HDC_ENC_FP32 && m->Fk == m->F) {
         *Xop = X;
@@ -177,7 +179,7 @@ hdc_status prepare_queries(const float *X, int64_t N, const hdc_model *m, char *
     const int ld = ld_for(m->enc, m->Fk);
     float *scale = m->enc == HDC_ENC_FP8_E4M3 ? (float *)(ws + L.sx) : nullptr;
     hdc_status s = cu(launch_quant_rows(X, m->F, 0, 1, N, m->Fk, m->enc, ws + L.xq, ld, scale, st, m->fs0,
-                                        m->fstride));
+                                        m->fstride, zero, zero_n));
     *Xop = ws + L.xq;
     *ldx = ld;
     *sx = scale;
@@ -491,10 +493,21 @@ hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m, int32_t *
         a.X = X; a.ldX = m->F; a.stage = (uint8_t *)ws + L.xq;
         if (tc_qin_ok(a) && tc_stage_bytes(a) <= (size_t)N * a.ldx * esize_for(m->enc)) return cu(timed_tc(a, st));
     }
+    // the fused classify of binary classes, and the scratch of a split batch
+    // (zeroed by the quantiser's launch)
+    TcArgs fused = {};
+    fused.N = N; fused.F = m->Fk; fused.ldx = ld_for(m->enc, m->Fk); fused.Bq = m->Bq; fused.ldb = m->ldb; fused.Dk = m->Dk;
+    fused.enc = m->enc; fused.sb = m->b_scale; fused.W = m->W;
+    fused.planes = m->cls; fused.C = m->C; fused.nb = nb; fused.csum = m->cls_sum; fused.cnorm = m->cls_norm;
+    fused.labels = labels; fused.dists = dists; fused.sims = scores;
+    fused.cls_sign = m->cls_sign; fused.ldcs = m->ldcs;
+    fused.dacc = (int32_t *)((char *)ws + L.dacc);
+    const bool fuse = use_tc(m) && !float_query(m->flags) && tc_supported(fused);
     const void *Xop;
     int64_t ldx;
     const float *sx;
-    hdc_status s = prepare_queries(X, N, m, (char *)ws, L, &Xop, &ldx, &sx, st);
+    hdc_status s = prepare_queries(X, N, m, (char *)ws, L, &Xop, &ldx, &sx, st, (uint32_t *)fused.dacc,
+                                   fuse ? tc_split_words(fused) : 0);
     if (s != HDC_OK) return s;
     uint32_t *Hb = (uint32_t *)((char *)ws + L.h);
     if (float_query(m->flags)) {
@@ -541,15 +554,10 @@ hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m, int32_t *
     }
     bool encoded = false;
     if (use_tc(m)) {
-        TcArgs a = {};
-        a.Xq = Xop; a.N = N; a.F = m->Fk; a.ldx = (int)ldx; a.Bq = m->Bq; a.ldb = m->ldb; a.Dk = m->Dk; a.enc = m->enc;
-        a.sx = sx; a.sb = m->b_scale; a.W = m->W;
-        a.planes = m->cls; a.C = m->C; a.nb = nb; a.csum = m->cls_sum; a.cnorm = m->cls_norm;
-        a.labels = labels; a.dists = dists; a.sims = scores;
-        a.cls_sign = m->cls_sign; a.ldcs = m->ldcs;
-        a.dacc = (int32_t *)((char *)ws + L.dacc);
+        TcArgs a = fused;
+        a.Xq = Xop; a.sx = sx;
         // binary classes: fully fused; otherwise tensor-core encode + K4
-        if (tc_supported(a)) return cu(timed_tc(a, st));
+        if (fuse) return cu(timed_tc(a, st));
         a.dacc = nullptr;
         TcArgs e = a;
         e.planes = nullptr; e.labels = nullptr; e.dists = nullptr; e.sims = nullptr; e.H = Hb;

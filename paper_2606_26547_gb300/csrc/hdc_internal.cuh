@@ -49,7 +49,8 @@ inline int esize_for(int enc) { return enc == HDC_ENC_BF16 ? 2 : enc == HDC_ENC_
 // (the kept features of a perforated encoding reduction).
 cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, int64_t row_step,
                               int64_t nrows, int F, int enc, void *dst, int ldd, float *scale,
-                              cudaStream_t st, int64_t c0 = 0, int64_t cstep = 1);
+                              cudaStream_t st, int64_t c0 = 0, int64_t cstep = 1, uint32_t *zero = nullptr,
+                              int64_t zero_n = 0);
 
 // Class preparation: planes [b][C][W] (or, with vals, the b-bit values as
 // BF16 rows of ldv elements, zero past Dk), sums and norms over the kept dims;
@@ -164,7 +165,8 @@ struct TcArgs {
     int64_t ldX;
     uint8_t *stage;
     // classify (binary classes, the popcount epilogue): scratch of
-    // tc_split_bytes(N, C) zero-filled per launch, so that a batch of few
+    // tc_split_bytes(N, C) whose first tc_split_words(a) words the caller has
+    // zeroed on the stream, so that a batch of few
     // query tiles can split each tile's dim tiles over several CTAs; NULL
     // keeps one CTA per query tile
     int32_t *dacc;
@@ -180,6 +182,10 @@ inline size_t tc_split_bytes(int64_t N, int C)
 }
 cudaError_t launch_tc_encode(const TcArgs &a, cudaStream_t st);
 bool tc_supported(const TcArgs &a);
+// Ranges the dim tiles of a classify's query tiles are split into (1: not
+// split), and the words of a.dacc such a launch needs zeroed.
+int tc_split(const TcArgs &a);
+int64_t tc_split_words(const TcArgs &a);
 // Whether the fused classify of a can quantise its own query tiles from the
 // FP32 rows a.X (binary classes: up to 32, or up to 112 with their E4M3
 // signs; 16-byte aligned rows of F % 4 == 0 floats; ldx <= 1024; at least two

@@ -166,6 +166,25 @@ size_t tc_stage_bytes(const TcArgs &a)
     return (size_t)2 * tc_grid(a.N, sms) * tc::BM * a.ldx * (a.enc == HDC_ENC_BF16 ? 2 : 1);
 }
 
+// A batch of fewer query tiles than SMs splits each tile's dim tiles so that
+// the batch fills the SMs (non-empty ranges only).
+int tc_split(const TcArgs &a)
+{
+    const int64_t m_tiles = (a.N + tc::BM - 1) / tc::BM;
+    const int sms = sm_count();
+    // the tensor-core Hamming kernel (33..112 classes) keeps whole tiles
+    if (!a.dacc || a.X || !a.planes || (a.cls_sign && a.C > 32 && a.C <= tc::H_CMAX) || m_tiles >= sms ||
+        m_tiles > TC_SPLIT_MAX_TILES)
+        return 1;
+    const int n_tiles = (a.Dk + tc::BN - 1) / tc::BN;
+    int ns = (int)(sms / m_tiles);
+    if (ns > n_tiles) ns = n_tiles;
+    const int per = (n_tiles + ns - 1) / ns;
+    return (n_tiles + per - 1) / per;
+}
+
+int64_t tc_split_words(const TcArgs &a) { return tc_split(a) > 1 ? a.N * a.C + (a.N + tc::BM - 1) / tc::BM : 0; }
+
 cudaError_t launch_tc_encode(const TcArgs &a, cudaStream_t st)
 {
     CUtensorMap ma, mb;
@@ -239,29 +258,16 @@ cudaError_t launch_tc_encode(const TcArgs &a, cudaStream_t st)
     }
     CUtensorMap mc = mb;  // unused by encode-only launches
     if (classify && !make_cls_map(&mc, a.planes, a.W, a.C)) return cudaErrorInvalidValue;
-    // few query tiles: split each tile's dim tiles over CTAs so that the
-    // batch fills the SMs (non-empty ranges only); partial distances meet
-    // in the zero-filled scratch
-    const int64_t m_tiles = (a.N + tc::BM - 1) / tc::BM;
-    const int n_tiles = (a.Dk + tc::BN - 1) / tc::BN;
-    unsigned g = grid;
-    if (classify && !qin && a.dacc && m_tiles < sms && m_tiles <= TC_SPLIT_MAX_TILES) {
-        int ns = (int)(sms / m_tiles);
-        if (ns > n_tiles) ns = n_tiles;
-        const int per = (n_tiles + ns - 1) / ns;
-        ns = (n_tiles + per - 1) / per;
-        if (ns > 1) {
-            p.nsplit = ns;
-            p.dacc = a.dacc;
-            p.tile_done = reinterpret_cast<unsigned *>(reinterpret_cast<char *>(a.dacc) +
-                                                       (size_t)a.N * a.C * 4);
-            const cudaError_t e = cudaMemsetAsync(a.dacc, 0, (size_t)a.N * a.C * 4 + (size_t)m_tiles * 4, st);
-            if (e != cudaSuccess) return e;
-            const int64_t units = m_tiles * ns;
-            g = (unsigned)(units < sms ? units : sms);
-        }
+    // few query tiles: each tile's dim tiles split over CTAs; partial
+    // distances meet in the zeroed scratch
+    const int ns = classify ? tc_split(a) : 1;
+    if (ns > 1) {
+        p.nsplit = ns;
+        p.dacc = a.dacc;
+        p.tile_done = reinterpret_cast<unsigned *>(a.dacc + a.N * a.C);
+        const int64_t units = (a.N + tc::BM - 1) / tc::BM * ns;
+        grid = (unsigned)(units < sms ? units : sms);
     }
-    grid = g;
     if (a.enc == HDC_ENC_BF16) return tc::launch_bf16(ma, mb, mc, p, grid, classify, st);
     return tc::launch_fp8(ma, mb, mc, p, grid, classify, st);
 }

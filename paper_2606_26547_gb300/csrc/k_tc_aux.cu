@@ -48,6 +48,8 @@ namespace {
 __global__ void class_bytes_kernel(const uint32_t *__restrict__ cls, int C, int W, int ldw, int64_t D, int64_t s0,
                                    int64_t e0, int64_t stride, uint32_t *__restrict__ out)
 {
+    // the packed kernel may be set up meanwhile (it waits for this one's end)
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (int64_t)C * ldw) return;
     const int c = (int)(i / ldw), x = (int)(i % ldw), w = x >> 3, j = x & 7;
@@ -115,13 +117,15 @@ cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensor
     lc.blockDim = dim3(tc::HP_THREADS);
     lc.dynamicSmemBytes = smem;
     lc.stream = st;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = (unsigned)pl.S;
-    at[0].val.clusterDim.y = 1;
-    at[0].val.clusterDim.z = 1;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = (unsigned)pl.S;
+    at[1].val.clusterDim.y = 1;
+    at[1].val.clusterDim.z = 1;
     lc.attrs = at;
-    lc.numAttrs = pl.S > 1 ? 1 : 0;
+    lc.numAttrs = pl.S > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&lc, k, p, mq, mc);
 }
 }  // namespace

@@ -82,6 +82,7 @@ __global__ void __launch_bounds__(192, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -248,8 +249,7 @@ cudaError_t launch_tc_cosine(const CosArgs &a, cudaStream_t st)
     cudaError_t e = cudaFuncSetAttribute(tc::tc_cosine_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)tc::CSMEM);
     if (e != cudaSuccess) return e;
-    tc::tc_cosine_kernel<<<grid, 192, tc::CSMEM, st>>>(ma, mb, p);
-    return cudaGetLastError();
+    return tc::launch_after(tc::tc_cosine_kernel, grid, 192, tc::CSMEM, st, ma, mb, p);
 }
 
 cudaError_t tc_cosine_read_status(cudaStream_t st, int *status) { return tc::read_status(st, status); }

@@ -151,6 +151,7 @@ __global__ void __launch_bounds__(FC_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -414,8 +415,7 @@ static cudaError_t launch_fcos_stages(const CUtensorMap &ma, const CUtensorMap &
     const size_t smem = fc_smem_bytes(STAGES, p.Cp, B2BUF);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, FC_THREADS, smem, st>>>(ma, mb, mv, p);
-    return cudaGetLastError();
+    return launch_after(k, grid, FC_THREADS, smem, st, ma, mb, mv, p);
 }
 
 template <int ENC>

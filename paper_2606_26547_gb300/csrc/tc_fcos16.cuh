@@ -135,6 +135,7 @@ __global__ void __launch_bounds__(F16_THREADS, 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -372,8 +373,7 @@ static cudaError_t launch_fcos16_enc(const CUtensorMap &ma, const CUtensorMap &m
     constexpr size_t smem = f16_smem_bytes<ENC>();
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, F16_THREADS, smem, st>>>(ma, mb, mv, ms, p);
-    return cudaGetLastError();
+    return launch_after(k, grid, F16_THREADS, smem, st, ma, mb, mv, ms, p);
 }
 
 cudaError_t launch_fcos16_bf16(const CUtensorMap &ma, const CUtensorMap &mb, const CUtensorMap &mv,

@@ -172,6 +172,7 @@ __global__ void __launch_bounds__(h_threads(QIN), 1)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    grid_wait();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -427,8 +428,7 @@ static cudaError_t launch_hamming_q(const CUtensorMap &ma, const CUtensorMap &mb
     const size_t smem = h_smem_bytes(p.Cp);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    k<<<grid, h_threads(QIN), smem, st>>>(ma, mb, ms, p);
-    return cudaGetLastError();
+    return launch_after(k, grid, h_threads(QIN), smem, st, ma, mb, ms, p);
 }
 
 template <int ENC>

@@ -286,6 +286,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    grid_wait();
     // class norms and their reciprocals, 0 for a zero norm (cosine, sweep: no
     // distances are staged there)
     double *s_norm = reinterpret_cast<double *>(s_out), *s_rinv = s_norm + HP_CMAX;
