@@ -115,8 +115,13 @@ def _ptr(t: torch.Tensor | None):
 
 
 def _stream(stream=None):
-    s = torch.cuda.current_stream() if stream is None else stream
-    return ctypes.c_void_p(s.cuda_stream)
+    if stream is None:
+        # the current stream's handle without a torch.cuda.Stream object around
+        # it: 0.2 us where current_stream() takes 3.0, a seventh of a one-row call
+        if torch.cuda.is_initialized():
+            return ctypes.c_void_p(torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice()))
+        stream = torch.cuda.current_stream()
+    return ctypes.c_void_p(stream.cuda_stream)
 
 
 @dataclasses.dataclass(frozen=True)
