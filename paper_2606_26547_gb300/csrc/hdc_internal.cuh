@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <initializer_list>
+
 #include "hdc.h"
 
 namespace hdc {
@@ -260,5 +262,41 @@ cudaError_t launch_tc_fcos(const TcArgs &a, const uint16_t *cv, int ldS, const d
 cudaError_t tc_cosine_read_status(cudaStream_t st, int *status);
 // Status word of the auxiliary tensor-core kernels (packed Hamming, wait self-test).
 cudaError_t tc_aux_read_status(cudaStream_t st, int *status);
+
+// Kernels that may be launched while the one before them in the stream still
+// runs (programmatic stream serialisation): early_wait returns when that kernel
+// is complete and its writes are visible, and lets the next launch start in
+// turn.  The pointers to what earlier kernels write pass through it: reads
+// through a const pointer are not ordered by the wait alone.
+template <typename P>
+__device__ __forceinline__ int read_after(P &p)
+{
+    asm volatile("" : "+l"(p)::"memory");
+    return 0;
+}
+
+template <typename... P>
+__device__ __forceinline__ void early_wait(P &...p)
+{
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    (void)std::initializer_list<int>{read_after(p)...};
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+template <typename... P, typename... A>
+cudaError_t launch_early(void (*k)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t st, bool early, A &&...args)
+{
+    cudaLaunchConfig_t c = {};
+    c.gridDim = grid;
+    c.blockDim = dim3(threads);
+    c.dynamicSmemBytes = smem;
+    c.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    c.attrs = &at;
+    c.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&c, k, P(args)...);
+}
 
 }  // namespace hdc

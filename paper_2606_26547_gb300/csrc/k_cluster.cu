@@ -135,8 +135,7 @@ __global__ void __launch_bounds__(STEP_ROWS * S) assign_count_kernel(const uint3
         smask[w] = m;
     }
     for (int i = tid; i < STEP_MAXK; i += T) s_cnt[i] = 0;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    early_wait(cls, lab);
     const int r = tid / S, s = tid % S;
     const bool own = s == 0 && r < nr;
     const int was = own && !first ? lab[n0 + r] : -1;
@@ -273,8 +272,7 @@ __global__ void __launch_bounds__(32 * UPD_SLICES) update_kernel(const uint32_t 
     __shared__ int32_t s_sum[UPD_SLICES][5][32];
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5, slices = blockDim.x >> 5, j = lane & 7;
     const int c = blockIdx.y, w = blockIdx.x * 4 + (lane >> 3);   // W is a multiple of 4
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;");
+    early_wait(planes, counts);
     const int32_t *cnt = counts + (int64_t)c * runs;
     // pairs of 16-bit sums: up to 64 for each of a warp's runs
     uint32_t lo = 0, hi = 0;
@@ -340,27 +338,12 @@ cudaError_t launch_step(const StepPlan &p, const uint32_t *H, int64_t N, int W, 
     cudaError_t e = cudaSuccess;
     if (first && p.smem > 40 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchAttribute early = {};
-    early.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    early.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t a = {};
-    a.gridDim = dim3((unsigned)p.runs);
-    a.blockDim = dim3((unsigned)(STEP_ROWS * p.S));
-    a.dynamicSmemBytes = p.smem;
-    a.stream = st;
-    a.attrs = &early;
-    a.numAttrs = first ? 0 : 1;
-    e = cudaLaunchKernelEx(&a, k, H, N, W, K, p.chunks, p.rows, p.words, p.runs, (const uint32_t *)cls,
-                           mask ? 1 : 0, mask ? mask->s0 : (int64_t)0, mask ? mask->e0 : (int64_t)0,
-                           mask ? mask->stride : (int64_t)1, lab, first, changes, planes, counts);
+    e = launch_early(k, dim3((unsigned)p.runs), (unsigned)(STEP_ROWS * p.S), p.smem, st, !first, H, N, W, K, p.chunks, p.rows,
+                     p.words, p.runs, cls, mask ? 1 : 0, mask ? mask->s0 : 0, mask ? mask->e0 : 0, mask ? mask->stride : 1,
+                     lab, first, changes, planes, counts);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t b = {};
-    b.gridDim = dim3((unsigned)(W / 4), (unsigned)K);
-    b.blockDim = dim3((unsigned)(32 * p.slices));
-    b.stream = st;
-    b.attrs = &early;
-    b.numAttrs = 1;
-    return cudaLaunchKernelEx(&b, update_kernel, (const uint32_t *)planes, (const int32_t *)counts, W, D, K, p.runs, acc, cls);
+    return launch_early(update_kernel, dim3((unsigned)(W / 4), (unsigned)K), (unsigned)(32 * p.slices), 0, st, true, planes,
+                        counts, W, D, K, p.runs, acc, cls);
 }
 
 struct ClusterLayout {

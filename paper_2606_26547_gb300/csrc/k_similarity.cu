@@ -269,7 +269,11 @@ __global__ void __launch_bounds__(TPB) hamming_csa_kernel(const uint32_t *__rest
         c2[c] = 0;
         d4[c] = 0;
     }
-    if (HIST && tid < 2 * CM) sh[tid] = 0;
+    if (HIST) {
+        // the grouping of the epoch's samples follows (early_wait)
+        asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+        if (tid < 2 * CM) sh[tid] = 0;
+    }
     const uint4 zero = make_uint4(0, 0, 0, 0);
     for (int w0 = 0; w0 < W; w0 += WC) {
         const int nw = min(WC, W - w0);   // a multiple of 4

@@ -55,6 +55,7 @@ __global__ void hist_kernel(const int32_t *__restrict__ y, const int32_t *__rest
                             int mode, int G, bool in_shared, int32_t *__restrict__ hist)
 {
     extern __shared__ int32_t sh[];
+    early_wait(y, pred, hist);
     int32_t *h = in_shared ? sh : hist;
     if (in_shared) {
         for (int g = threadIdx.x; g < G; g += blockDim.x) sh[g] = 0;
@@ -80,6 +81,7 @@ __global__ void scan_kernel(const int32_t *__restrict__ hist, int G, int C, int3
                             int32_t *__restrict__ items, int32_t *__restrict__ cursor,
                             int32_t *__restrict__ n_updates)
 {
+    early_wait(hist);
     if (threadIdx.x != 0) return;
     int32_t s = 0, it = 0;
     for (int g = 0; g < G; g++) {
@@ -153,6 +155,7 @@ __global__ void __launch_bounds__(256) scatter_kernel(const int32_t *__restrict_
     __shared__ int32_t s_off[SEG_SMEM_G + 1];
     __shared__ int32_t s_cnt[SEG_SMEM_G];
     __shared__ int32_t s_base[SEG_SMEM_G];
+    early_wait(y, pred, hist, offsets_in, cursor);
     const int64_t n0 = (int64_t)blockIdx.x * run;
     const int64_t n1 = min(N, n0 + run);
     if (hist) {
@@ -250,6 +253,7 @@ __global__ void __launch_bounds__(TW) count_kernel(const uint32_t *__restrict__ 
     __shared__ int32_t s_rows[CH];
     __shared__ int32_t s_off[SEG_SMEM_G + 1];
     __shared__ int32_t s_items[SEG_SMEM_G + 1];
+    early_wait(H, perm, hist, offsets, items);
     const bool small = G <= SEG_SMEM_G;
     if (small) {
         warp_scan_groups(hist, G, s_off, s_items);
@@ -338,6 +342,7 @@ __global__ void __launch_bounds__(32 * RED_SLICES) reduce_kernel(const uint32_t 
                                                                  uint32_t *__restrict__ cls)
 {
     __shared__ int32_t s_sum[RED_SLICES][4][32];
+    early_wait(partial, offsets, items);
     const int lane = threadIdx.x & 31, slice = threadIdx.x >> 5;
     const int64_t t = (int64_t)blockIdx.x * 32 + lane;
     const bool live = t < (int64_t)C * W * 8;
@@ -434,19 +439,28 @@ cudaError_t group_and_count(const uint32_t *H, int W, const int32_t *y, const in
     int64_t blocks = (N + 255) / 256;
     if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;
     if (blocks < 1) blocks = 1;
+    // hist_kernel follows a memset or a prediction; the kernels after it start
+    // while their predecessor ends and wait for it (early_wait): the four to
+    // five launches of a pass are short, their set-up a part of each
+    cudaError_t e = cudaSuccess;
     if (!hist_ready) {
         const bool in_shared = (size_t)G * sizeof(int32_t) <= 48 * 1024;
-        hist_kernel<<<(unsigned)blocks, 256, in_shared ? (size_t)G * sizeof(int32_t) : 0, st>>>(y, pred, N, C, mode,
-                                                                                                G, in_shared, s.hist);
+        e = launch_early(hist_kernel, dim3((unsigned)blocks), 256, in_shared ? (size_t)G * sizeof(int32_t) : 0, st, false, y,
+                         pred, N, C, mode, G, in_shared, s.hist);
+        if (e != cudaSuccess) return e;
     }
     // up to SEG_SMEM_G groups the scatter and counting kernels scan the
     // histogram themselves; the cursors were zeroed with it
     const bool small = G <= SEG_SMEM_G;
-    if (!small) scan_kernel<<<1, 32, 0, st>>>(s.hist, G, C, s.offsets, s.items, s.cursor, n_updates);
+    if (!small) {
+        e = launch_early(scan_kernel, dim3(1), 32, 0, st, true, s.hist, G, C, s.offsets, s.items, s.cursor, n_updates);
+        if (e != cudaSuccess) return e;
+    }
     int64_t run = (N + (int64_t)sms * 4 - 1) / ((int64_t)sms * 4);
     run = (run + 255) / 256 * 256;
-    scatter_kernel<<<(unsigned)((N + run - 1) / run), 256, 0, st>>>(y, pred, N, run, C, mode, small ? s.hist : nullptr,
-                                                                   G, s.offsets, s.cursor, s.perm);
+    e = launch_early(scatter_kernel, dim3((unsigned)((N + run - 1) / run)), 256, 0, st, true, y, pred, N, run, C, mode,
+                     small ? s.hist : nullptr, G, s.offsets, s.cursor, s.perm);
+    if (e != cudaSuccess) return e;
     // items: at most ceil(entries / CH) + G, entries <= (G / C) * N; one
     // block per (item, word block), extra grid rows exit at once
     const int64_t max_items = train_max_items(N, C);
@@ -455,16 +469,12 @@ cudaError_t group_and_count(const uint32_t *H, int W, const int32_t *y, const in
     int64_t rows = max_items < 65535 ? max_items : 65535;
     const dim3 grid((unsigned)wblocks, (unsigned)rows);
     int32_t *nu = small ? n_updates : nullptr;
-    if (wtile == 128)
-        count_kernel<128><<<grid, 128, 0, st>>>(H, W, s.perm, s.hist, s.offsets, s.items, G, C, nu, s.partial);
-    else if (wtile == 64)
-        count_kernel<64><<<grid, 64, 0, st>>>(H, W, s.perm, s.hist, s.offsets, s.items, G, C, nu, s.partial);
-    else
-        count_kernel<32><<<grid, 32, 0, st>>>(H, W, s.perm, s.hist, s.offsets, s.items, G, C, nu, s.partial);
+    auto count = wtile == 128 ? count_kernel<128> : wtile == 64 ? count_kernel<64> : count_kernel<32>;
+    e = launch_early(count, grid, (unsigned)wtile, 0, st, true, H, W, s.perm, s.hist, s.offsets, s.items, G, C, nu, s.partial);
+    if (e != cudaSuccess) return e;
     const int64_t threads = (int64_t)C * W * 8;
-    reduce_kernel<<<(unsigned)((threads + 31) / 32), 32 * RED_SLICES, 0, st>>>(s.partial, W, D, s.offsets, s.items, G, C,
-                                                                      accumulate, acc, cls);
-    return cudaGetLastError();
+    return launch_early(reduce_kernel, dim3((unsigned)((threads + 31) / 32)), 32 * RED_SLICES, 0, st, true, s.partial, W, D,
+                        s.offsets, s.items, G, C, accumulate, acc, cls);
 }
 
 }  // namespace
