@@ -104,7 +104,7 @@ cudaError_t launch_argmin_groups(const uint32_t *H, int64_t N, const uint32_t *c
 // Scratch (train_max_items(N, C) counting items): perm (2N int32), hist and
 // cursor (2C int32), offsets and items (2C + 1 int32), partial (max items x
 // W x 8 uint32 byte lanes).
-// signs: for 33..256 classes, Cp x hamming_packed_ldcs(W) bytes for the
+// signs: for 17..256 classes, Cp x hamming_packed_ldcs(W) bytes for the
 // class hypervectors expanded once per epoch (NULL: the Hamming kernel
 // expands them itself).
 struct TrainScratch {
@@ -112,13 +112,15 @@ struct TrainScratch {
     uint32_t *partial;
     uint8_t *signs;
 };
-// Bytes of the expanded class hypervectors the training and clustering
-// workspaces hold (0 outside 33..256 classes).
+// Bytes of the expanded class hypervectors: in the caller's Hamming workspace
+// (0 outside 33..256 classes, as its size is published), and in the training and
+// clustering workspaces (0 outside 17..256).
 size_t class_sign_bytes(int C, int W);
+size_t scratch_sign_bytes(int C, int W);
 // Hamming arg-min of N packed rows against C classes over the kept dims
 // (s0, s0 + stride, ... < e0; all of [0, D) for a stride-1 full range): the
 // library's routes, with the class hypervectors expanded into `signs`
-// (class_sign_bytes(C, W), or NULL) for the tensor-core route.
+// (scratch_sign_bytes(C, W), or NULL) for the tensor-core route.
 cudaError_t launch_argmin_ws(const uint32_t *H, int64_t N, const uint32_t *cls, int C, int W, int64_t D,
                              const Perf *p, int32_t *labels, uint8_t *signs, cudaStream_t st);
 int64_t train_max_items(int64_t N, int C);
@@ -200,6 +202,8 @@ size_t tc_stage_bytes(const TcArgs &a);
 // Reads and clears the streaming quantiser's device status word.
 cudaError_t quant_read_status(cudaStream_t st, int *status);
 
+// Most rows of the tensor-core Hamming kernel (32-bit row coordinates).
+constexpr int64_t kMaxPackedRows = 0x7fffffffLL - 256;
 // Reads and clears the tensor-core kernels' device status word.
 cudaError_t tc_read_status(cudaStream_t st, int *status);
 // Hamming arg-min of packed rows on the tensor cores (up to 256 binary

@@ -357,8 +357,8 @@ bool cluster_layout(int64_t N, int D, int K, ClusterLayout *L)
     size_t off = 0;
     L->lab0 = off;  off = align_up(off + (size_t)N * 4, kAlign);
     L->lab1 = off;  off = align_up(off + (size_t)N * 4, kAlign);
-    // the cluster hypervectors expanded to bytes for the assignment (K > 32)
-    L->signs = off; off = align_up(off + class_sign_bytes(K, words_for(D)), kAlign);
+    // the cluster hypervectors expanded to bytes for the assignment (K > 16)
+    L->signs = off; off = align_up(off + scratch_sign_bytes(K, words_for(D)), kAlign);
     L->train = off; off = align_up(off + tb, kAlign);
     const StepPlan p = step_plan(N, words_for(D), K);
     L->planes = off;
@@ -415,7 +415,7 @@ extern "C" hdc_status hdc_cluster(const uint32_t *H, int64_t N, int32_t D, int32
     cudaStream_t st = (cudaStream_t)stream;
     char *w = (char *)ws;
     int32_t *lab[2] = {(int32_t *)(w + L.lab0), (int32_t *)(w + L.lab1)};
-    uint8_t *signs = class_sign_bytes(K, words_for(D)) ? (uint8_t *)(w + L.signs) : nullptr;
+    uint8_t *signs = scratch_sign_bytes(K, words_for(D)) ? (uint8_t *)(w + L.signs) : nullptr;
     const int W = words_for(D);
     Perf pt, pi;
     const Perf *ptrain = perf_or_null(D, train_sim, &pt), *pinfer = perf_or_null(D, infer_sim, &pi);

@@ -462,14 +462,16 @@ cudaError_t launch_similarity(const uint32_t *Q, int64_t N, const uint32_t *plan
                                               nullptr, st);
         return launch_csa<false, false>(Q, N, planes, C, W, 0, D, 1, labels, dists, nullptr, nullptr, st);
     }
-    if (nb == 1 && C <= 32) return launch_reg<32>(Q, N, planes, C, W, D, p, labels, dists, st);
-    // 33..256 binary classes: the distances as a tensor-core product of the
-    // rows expanded to +-1 (the popcount loop is bound by the popcount unit,
-    // ~16 per clock per SM; up to 32 classes it measured faster, the
-    // expansion not yet amortised: 0.24 vs 0.35 ms for 10^6 x 1,024 dims x 26)
-    if (nb == 1 && C > 32 && hamming_packed_ok(C, W))
+    // 17..256 binary classes: the distances as a tensor-core product of the
+    // rows expanded to +-1, whose time hardly depends on the classes where the
+    // popcount loop is bound by the popcount unit (~16 per clock per SM).
+    // 100,000 x 16,384 dims x 32: 193 us, popcounts 428; 10,000 x 4,096 x 17:
+    // 15.6 / 22.9; equal where a launch's latency is all (300 x 1,024).  Up to
+    // 16 classes the carry-save kernel above is the faster (x 16: 160 / 191).
+    if (nb == 1 && hamming_packed_ok(C, W) && (C > 32 || N <= kMaxPackedRows))
         return launch_hamming_packed(Q, N, planes, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      dists, st);
+    if (nb == 1 && C <= 32) return launch_reg<32>(Q, N, planes, C, W, D, p, labels, dists, st);
     if (nb == 1) return launch_reg<64>(Q, N, planes, C, W, D, p, labels, dists, st);   // chunks of 64 classes
     switch (nb) {
     case 1: return launch_nb<1>(Q, N, planes, C, W, D, p, csum, cnorm, labels, dists, scores, st);

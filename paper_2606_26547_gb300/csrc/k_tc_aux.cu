@@ -146,7 +146,7 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
                                   cudaStream_t st, uint8_t *signs)
 {
     if (N <= 0) return cudaSuccess;
-    if (!hamming_packed_ok(C, W) || stride < 1 || N > 0x7fffffffLL - 2 * tc::BM) return cudaErrorNotSupported;
+    if (!hamming_packed_ok(C, W) || stride < 1 || N > kMaxPackedRows) return cudaErrorNotSupported;
     const int ldcs = hamming_packed_ldcs(W), R = (C + 15) / 16 * 16;
     CUtensorMap mq, mc;
     if (!make_packed_map(&mq, Q, W, N)) return cudaErrorInvalidValue;

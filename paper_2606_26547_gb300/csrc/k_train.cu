@@ -531,7 +531,14 @@ cudaError_t launch_binarise(const int32_t *acc, int C, int D, uint32_t *cls, int
 
 size_t class_sign_bytes(int C, int W)
 {
-    if (C <= 32 || !hamming_packed_ok(C, W)) return 0;
+    return C <= 32 ? 0 : scratch_sign_bytes(C, W);
+}
+
+// Expanded once instead of by every tile (100,000 x 16,384 x 32: 117 us, 193
+// without, popcounts 428).
+size_t scratch_sign_bytes(int C, int W)
+{
+    if (C <= 16 || !hamming_packed_ok(C, W)) return 0;
     return (size_t)((C + 15) / 16 * 16) * hamming_packed_ldcs(W);
 }
 
@@ -539,7 +546,7 @@ cudaError_t launch_argmin_ws(const uint32_t *H, int64_t N, const uint32_t *cls, 
                              const Perf *p, int32_t *labels, uint8_t *signs, cudaStream_t st)
 {
     if (N <= 0) return cudaSuccess;
-    if (signs && class_sign_bytes(C, W) > 0) {
+    if (signs && scratch_sign_bytes(C, W) > 0) {
         // expand the classes once, then stream them to the tensor-core route
         return launch_hamming_packed(H, N, cls, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      nullptr, st, signs);
