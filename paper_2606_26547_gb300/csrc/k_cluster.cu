@@ -50,13 +50,13 @@ constexpr int CHIP_SMS = 152;
 
 // Lines of the route, from both sides timed (us an iteration, 2 / 7 launches): a
 // block's planes are K W words a plane, so runs * K * W bounds the traffic
-// (8,000 x 10,000 x 26, 1.0 M: 53 / 76; 8,000 x 10,000 x 64, 2.6 M: 112 / 74;
-// 20,000 x 4,096 x 26, 1.0 M: 62 / 59) and K * W the time of one block (500 x
-// 10,000 x 26, 8,320: 32 / 64; x 64, 20,480: 64 / 69).  Past one block an SM the
-// row copies count as well (20,000 x 512 x 26: 18 / 37; 20,000 x 10,000 x 4:
-// 60 / 43; 60,000 x 512 x 4: 50 / 34).  Eight threads a point while the blocks
-// fit one to an SM, four in two resident blocks beyond (20,000 x 1,024 x 26:
-// 25.5 / 21.5; 8,000: 10.5 / 13.6).
+// (9,700 x 4,096 x 26, 506 K: 28 / 36; 5,000 x 6,000 x 36, 535 K: 40 / 37;
+// 16,000 x 2,048 x 50, 800 K: 44 / 37), K * W the time of one block (500 x 6,000 x
+// 50, 9,400: 38 / 37; 500 x 10,000 x 26, 8,320: 33 / 36), N * W the copies of the
+// rows (9,700 x 6,000 x 16, 1.8 M: 29 / 34; 16,000 x 4,096 x 10, 2.0 M: 34 / 32;
+// 9,700 x 10,000 x 4, 3.1 M: 34 / 31).  Eight threads a point while the blocks fit
+// one to an SM, four in two resident blocks beyond (20,000 x 1,024 x 26: 25.5 /
+// 21.5; 8,000: 10.5 / 13.6).
 struct StepPlan {
     bool ok;
     int S;             // threads a point
@@ -70,9 +70,10 @@ struct StepPlan {
 StepPlan step_plan(int64_t N, int W, int K)
 {
     StepPlan p = {};
-    if (N <= 0 || N > 16384 || K > STEP_MAXK || (int64_t)K * W > 12288) return p;
+    if (N <= 0 || N > 16384 || K > STEP_MAXK || (int64_t)K * W > 9000 || N * W > 1850000)
+        return p;
     p.runs = (int)((N + STEP_ROWS - 1) / STEP_ROWS);
-    if ((int64_t)p.runs * K * W > 1000000 || (p.runs > CHIP_SMS && W > 128)) return p;
+    if ((int64_t)p.runs * K * W > 520000) return p;
     p.S = p.runs <= CHIP_SMS && W >= 32 ? 8 : 4;
     p.chunks = K > 32 ? 2 : 1;
     p.cm = ((K + p.chunks - 1) / p.chunks + 7) / 8 * 8;

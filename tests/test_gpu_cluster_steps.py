@@ -14,14 +14,16 @@ torch = pytest.importorskip("torch")
 # block's 64 and the update's 16 parts of the runs; words of a part of a 16-word
 # step and of a 32-word chunk; every point of a block in one cluster (K = 1);
 # kept dims; one block an SM (9,728 points) and past it; past each line of the
-# route (16,384 points, clusters x words, blocks x clusters x words)
+# route (16,384 points, clusters x words, blocks x clusters x words, points x words)
 @pytest.mark.parametrize("N,D,K,tp", [
     (1, 33, 1, (0.0, 1.0, 1)), (64, 128, 1, (0.0, 1.0, 1)), (65, 500, 8, (0.1, 0.8, 1)), (200, 513, 9, (0.0, 1.0, 3)),
     (1024, 1025, 26, (0.0, 1.0, 1)), (1025, 2100, 32, (0.0, 1.0, 2)), (1500, 4096, 33, (0.3, 1.0, 1)),
     (2500, 640, 64, (0.0, 1.0, 1)), (700, 640, 65, (0.0, 1.0, 1)), (9728, 1024, 3, (0.0, 1.0, 1)),
     (9729, 1030, 26, (0.0, 0.9, 1)), (16384, 96, 5, (0.0, 1.0, 1)), (16385, 96, 5, (0.0, 1.0, 1)),
     (9729, 4200, 2, (0.0, 1.0, 1)), (90, 40000, 9, (0.0, 1.0, 1)), (90, 40000, 10, (0.0, 1.0, 1)),
-    (9700, 4096, 54, (0.0, 1.0, 1)), (9700, 4096, 53, (0.0, 1.0, 1))])
+    (9700, 4096, 54, (0.0, 1.0, 1)), (9700, 4096, 53, (0.0, 1.0, 1)), (9700, 4096, 27, (0.0, 1.0, 1)),
+    (9700, 4096, 26, (0.0, 1.0, 1)), (90, 40000, 8, (0.0, 1.0, 1)), (90, 40000, 7, (0.0, 1.0, 1)),
+    (9728, 6100, 3, (0.0, 1.0, 1)), (9600, 6100, 3, (0.0, 1.0, 1))])
 def test_iterations(N, D, K, tp):
     from paper_2606_26547_gb300 import hdc
     rng = np.random.default_rng(N + D + K)
