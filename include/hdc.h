@@ -201,9 +201,10 @@ hdc_status hdc_hamming_argmin(const uint32_t *Q, const uint32_t *Cls,
                               int32_t *dists, hdc_stream_t stream);
 
 /* Workspace bytes for hdc_hamming_argmin_ws: for 33..256 classes and
- * D <= 131072 (the tensor-core route), the class hypervectors expanded to
+ * D <= 131072 (on the tensor-core route), the class hypervectors expanded to
  * one E4M3 +-1 byte per dim (C rounded up to 16 rows of
- * 256 * ceil(W(D) / 8) bytes); 0 for every other C and D.
+ * 256 * ceil(W(D) / 8) bytes); 0 for every other C and D (17..32 classes
+ * take that route without one).
  * HDC_ERR_INVALID_ARG for C <= 0, D <= 0 or a NULL bytes.                  */
 hdc_status hdc_hamming_argmin_workspace_bytes(int32_t C, int32_t D, size_t *bytes);
 
