@@ -96,10 +96,9 @@ __device__ __forceinline__ void cp16(void *dst, const void *src, bool on)
 
 // Block b: the points from 64 b.  S threads share a point: thread s takes
 // the words 4 s .. 4 s + 3 of every 4 S, 16 bytes of the point and of each
-// cluster hypervector at a time.  The differing bits of the four words are added
-// to a carry-save pair per cluster before they are counted: POPC runs at a
-// quarter of the rate of the logic.  planes[((b K + c) 7 + p) W + w];
-// counts[c runs + b].
+// cluster hypervector at a time.  The differing bits of the four words pass two
+// full adders per cluster before the carries are counted (hamming_csa_kernel).
+// planes[((b K + c) 7 + p) W + w]; counts[c runs + b].
 template <int CM, int S>
 __global__ void __launch_bounds__(STEP_ROWS * S) assign_count_kernel(const uint32_t *__restrict__ H, int64_t N, int W, int K,
                                                               int chunks, int P, int Wp, int runs,
@@ -151,10 +150,10 @@ __global__ void __launch_bounds__(STEP_ROWS * S) assign_count_kernel(const uint3
 
     int best = 0x7fffffff;   // distance * 64 + cluster: the lowest index on ties
     for (int cb = 0; cb < KP; cb += CM) {
-        uint32_t ones[CM], twos[CM];
+        uint32_t ones[CM];
         int dist[CM];
 #pragma unroll
-        for (int c = 0; c < CM; c++) ones[c] = twos[c] = 0, dist[c] = 0;
+        for (int c = 0; c < CM; c++) ones[c] = 0, dist[c] = 0;
         for (int w = 4 * s; w < Wp; w += 4 * S) {
             const uint4 q = *reinterpret_cast<const uint4 *>(srow + r * P + w);
             const uint4 m = *reinterpret_cast<const uint4 *>(smask + w);
@@ -163,17 +162,16 @@ __global__ void __launch_bounds__(STEP_ROWS * S) assign_count_kernel(const uint3
             for (int c = 0; c < CM; c++) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(cw + c * Wp);
                 const uint32_t x0 = (q.x ^ v.x) & m.x, x1 = (q.y ^ v.y) & m.y, x2 = (q.z ^ v.z) & m.z, x3 = (q.w ^ v.w) & m.w;
-                uint32_t &a = ones[c], &b = twos[c];
+                uint32_t &a = ones[c];
                 const uint32_t y0 = (a & x0) | (x1 & (a | x0));
                 a ^= x0 ^ x1;
                 const uint32_t y1 = (a & x2) | (x3 & (a | x2));
                 a ^= x2 ^ x3;
-                dist[c] += __popc((b & y0) | (y1 & (b | y0)));
-                b ^= y0 ^ y1;
+                dist[c] += __popc(y0) + __popc(y1);
             }
         }
 #pragma unroll
-        for (int c = 0; c < CM; c++) dist[c] = 4 * dist[c] + 2 * __popc(twos[c]) + __popc(ones[c]);
+        for (int c = 0; c < CM; c++) dist[c] = 2 * dist[c] + __popc(ones[c]);
         // sums over the S threads; each ends with a quarter (S = 4) or an eighth
         // of the clusters
         int h[CM / 2], t[CM / 4];

@@ -238,10 +238,11 @@ __device__ __forceinline__ uint32_t perf_word_mask(int64_t w, int64_t s0, int64_
 // The class words of a chunk of WC words sit in shared memory (zero past C;
 // both the class words and the query words are ANDed with the kept-dim mask,
 // so (q ^ c) counts only kept dims).  Per class, the four mismatch words
-// x = q ^ c enter a bit-sliced carry-save counter of planes of weight 1 and
-// 2 (three full adders); only the carry of weight 4 is popcounted, one
-// popcount per four words instead of four, the remaining work being 3-input
-// logic operations.  dist = 4 * sum popc(e4) + 2 popc(c2) + popc(c1), summed
+// x = q ^ c pass two full adders with a bit-sliced plane of weight 1, and the two
+// carries of weight 2 are popcounted: 9 operations on the logic pipe (two clocks
+// a warp each) beside two popcounts on a pipe of their own (eight each), 18 and
+// 16 clocks.  A third adder and one popcount (22 and 8) took 44.5 us where this
+// takes 39.4 (60,000 x 10,000 x 10); dist = 2 * sum popc(e2) + popc(c1), summed
 // over the four threads by shuffles.  With HIST, the kernel also counts the
 // groups of a retraining epoch: a sample whose prediction differs from its
 // label y goes to group y (added) and group C + prediction (subtracted).
@@ -261,13 +262,12 @@ __global__ void __launch_bounds__(TPB) hamming_csa_kernel(const uint32_t *__rest
     const int64_t row = (int64_t)blockIdx.x * (TPB / 4) + (tid >> 2);
     const bool valid = row < N;
     const uint32_t *q = Q + (valid ? row : 0) * (int64_t)W;
-    uint32_t c1[CM], c2[CM];
-    int d4[CM];
+    uint32_t c1[CM];
+    int d2[CM];
 #pragma unroll
     for (int c = 0; c < CM; c++) {
         c1[c] = 0;
-        c2[c] = 0;
-        d4[c] = 0;
+        d2[c] = 0;
     }
     if (HIST) {
         // the grouping of the epoch's samples follows (early_wait)
@@ -323,11 +323,10 @@ __global__ void __launch_bounds__(TPB) hamming_csa_kernel(const uint32_t *__rest
 #pragma unroll
             for (int c = 0; c < CM; c++) {
                 const uint4 v = *reinterpret_cast<const uint4 *>(sc + c * WC + j);
-                uint32_t a2, b2, e4;
+                uint32_t a2, b2;
                 csa(a2, c1[c], c1[c], qv.x ^ v.x, qv.y ^ v.y);
                 csa(b2, c1[c], c1[c], qv.z ^ v.z, qv.w ^ v.w);
-                csa(e4, c2[c], c2[c], a2, b2);
-                d4[c] += __popc(e4);
+                d2[c] += __popc(a2) + __popc(b2);
             }
         }
         cp_async_wait<0>();   // the ring's trailing zero-fills land before the next chunk reuses it
@@ -335,7 +334,7 @@ __global__ void __launch_bounds__(TPB) hamming_csa_kernel(const uint32_t *__rest
     int best = 0, bv = 0x7fffffff;
 #pragma unroll
     for (int c = 0; c < CM; c++) {
-        int v = 4 * d4[c] + 2 * __popc(c2[c]) + __popc(c1[c]);
+        int v = 2 * d2[c] + __popc(c1[c]);
         v += __shfl_xor_sync(0xffffffffu, v, 1);
         v += __shfl_xor_sync(0xffffffffu, v, 2);
         if (c < C) {
