@@ -15,7 +15,7 @@
 // between them).  ID and level rows are compacted to the kept dims at
 // model preparation, like the base rows of the random projection.
 //
-// Encode kernel of small batches: one block per (32 queries, 32 words); the block stages its
+// Encode kernel of medium batches: one block per (32 queries, 32 words); the block stages its
 // word slice of every ID row and every level row in shared memory.  A warp
 // takes four queries at a time (four independent counter chains, each ID
 // word loaded once for the four), a lane one word (32 dims): lane j
@@ -241,6 +241,77 @@ __global__ void __launch_bounds__(LWARPS * 32) levelid_encode_kernel(const float
         }
         tile += gridDim.x;
     } while (REST && tile * LQ < N);
+}
+
+// ---- few queries ------------------------------------------------------------
+//
+// One wave of the kernel above is latency: the rows staged a load at a time, then
+// 32 features after another whose values come from device memory, in one warp
+// where there are four queries.  Here the rows are staged by asynchronous
+// copies while all of the queries' levels are formed, and a warp takes Q1
+// queries: one while the blocks fit the SMs, four then.  One query, 561 x 4,928,
+// 128 levels 48 -> 15 us; 1,000, 617 x 1,024 62 -> 19 (four a warp, 3,000: 64 -> 54).
+template <int HP, int Q1>
+__global__ void __launch_bounds__(LWARPS * 32) levelid_few_kernel(const float *__restrict__ X, int64_t N, int F, int L, int W,
+                                                                float lo, float scale, const uint32_t *__restrict__ id,
+                                                                const uint32_t *__restrict__ lv, uint32_t *__restrict__ H)
+{
+    extern __shared__ __align__(16) uint32_t lsm[];
+    const uint32_t *sid = lsm, *slv = lsm + (size_t)F * LWC;         // F x LWC, L x LWC
+    const int Fp = (F + 3) / 4 * 4;
+    int *soff = reinterpret_cast<int *>(lsm + (size_t)(F + L) * LWC);   // [LWARPS * Q1][Fp] level-row offsets
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int w0 = blockIdx.y * LWC, nw = min(LWC, W - w0);          // W is a multiple of 4
+    for (int i = threadIdx.x; i < (F + L) * (LWC / 4); i += LWARPS * 32) {
+        const int r = i / (LWC / 4), c = i % (LWC / 4) * 4;
+        const uint32_t *src = (r < F ? id + (int64_t)r * W : lv + (int64_t)(r - F) * W) + w0 + c;
+        const uint32_t dst = (uint32_t)__cvta_generic_to_shared(lsm + r * LWC + c);
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst), "l"(c < nw ? src : id), "r"(c < nw ? 16 : 0));
+    }
+    asm volatile("cp.async.commit_group;");
+    const int64_t q0 = ((int64_t)blockIdx.x * LWARPS + warp) * Q1;   // this warp's queries
+    int *off = soff + warp * Q1 * Fp;
+#pragma unroll
+    for (int a = 0; a < Q1; a++)
+#pragma unroll 8
+        for (int f = lane; f < F; f += 32)
+            off[a * Fp + f] = q0 + a < N ? quant_level(__ldg(X + (q0 + a) * F + f), lo, scale, L) * LWC : 0;
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncthreads();
+    if (q0 >= N) return;
+    Counter<HP> cnt[Q1];
+#pragma unroll
+    for (int a = 0; a < Q1; a++) {
+        cnt[a].c1 = cnt[a].c2 = cnt[a].c4 = cnt[a].c8 = 0;
+#pragma unroll
+        for (int k = 0; k < HP; k++) cnt[a].hp[k] = 0;
+    }
+    int f = 0;
+    for (; f + 16 <= F; f += 16) {
+        uint32_t idw[16];
+#pragma unroll
+        for (int u = 0; u < 16; u++) idw[u] = sid[(f + u) * LWC + lane];
+#pragma unroll
+        for (int a = 0; a < Q1; a++) {
+            const int4 *o4 = reinterpret_cast<const int4 *>(off + a * Fp + f);
+            uint32_t r[16];
+#pragma unroll
+            for (int v = 0; v < 4; v++) {
+                const int4 t = o4[v];
+                r[4 * v] = idw[4 * v] ^ slv[t.x + lane];
+                r[4 * v + 1] = idw[4 * v + 1] ^ slv[t.y + lane];
+                r[4 * v + 2] = idw[4 * v + 2] ^ slv[t.z + lane];
+                r[4 * v + 3] = idw[4 * v + 3] ^ slv[t.w + lane];
+            }
+            add16(cnt[a], r);
+        }
+    }
+    for (; f < F; f++)
+#pragma unroll
+        for (int a = 0; a < Q1; a++) add1(cnt[a], sid[f * LWC + lane] ^ slv[off[a * Fp + f] + lane]);
+#pragma unroll
+    for (int a = 0; a < Q1; a++)
+        if (q0 + a < N && lane < nw) H[(q0 + a) * (int64_t)W + w0 + lane] = greater(cnt[a], (uint32_t)F >> 1);
 }
 
 // ---- many queries ----------------------------------------------------------
@@ -688,6 +759,19 @@ extern "C" hdc_status hdc_levelid_encode(const float *X, int64_t N, const hdc_le
                  : m->F <= 640 ? launch_count<20>(X, N, *m, H, slices, st)
                                : launch_count<25>(X, N, *m, H, slices, st)) != cudaSuccess)
         return HDC_ERR_CUDA;
+    // one and four queries a warp where that is a wave of one block an SM
+    for (int q1 = 1; q1 <= 4 && !many; q1 += 3) {
+        const int64_t blocks = (N + LWARPS * q1 - 1) / (LWARPS * q1);
+        const size_t smem = encode_smem(m->F, m->L) + (size_t)LWARPS * q1 * ((m->F + 3) / 4 * 4) * 4;
+        if (blocks * slices > SMS || smem > 220 * 1024 || (((uintptr_t)m->id | (uintptr_t)m->level) & 15)) continue;
+        auto k = hp_for(m->F) == 6 ? (q1 == 1 ? levelid_few_kernel<6, 1> : levelid_few_kernel<6, 4>)
+                                   : (q1 == 1 ? levelid_few_kernel<9, 1> : levelid_few_kernel<9, 4>);
+        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
+            return HDC_ERR_CUDA;
+        k<<<dim3((unsigned)blocks, (unsigned)slices), LWARPS * 32, smem, st>>>(X, N, m->F, m->L, m->W, m->lo, m->scale, m->id,
+                                                                              m->level, H);
+        return cudaGetLastError() == cudaSuccess ? HDC_OK : HDC_ERR_CUDA;
+    }
     const size_t smem = encode_smem(m->F, m->L) + LOFF_BYTES;
     // counter planes for floor(F / 16) (F < 8192: at most 9)
     auto k = hp_for(m->F) != 6 ? levelid_encode_kernel<9, false>

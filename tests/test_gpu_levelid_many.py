@@ -79,6 +79,22 @@ def test_many(hdc, F, D, L, N, ends):
     assert np.array_equal(unpack(out[pick].cpu().numpy().view(np.uint32), D), ref)
 
 
+# few queries: one and four a warp and the rows' kernel past them; features around
+# the 16-row groups and the counter's planes (1,024); part words, several slices
+@pytest.mark.parametrize("F,D,L,N", [(1, 33, 2, 1), (15, 100, 5, 8), (16, 1024, 7, 9), (35, 1030, 130, 300),
+                                     (20, 100, 5, 1216), (20, 100, 5, 1217), (21, 130, 5, 4864), (20, 100, 5, 4865),
+                                     (617, 1024, 128, 11), (1030, 200, 20, 3), (1030, 200, 20, 1300), (1500, 70, 60, 5)])
+def test_few(hdc, F, D, L, N):
+    hvs, g = make(hdc, F, D, L, "random", N + F)
+    m = hdc.LevelIdModel(*hvs, L, -2.0, 2.5)
+    X = torch.randn((N, F), generator=g, device="cuda") * 1.5
+    X[0, 0], X[N - 1, F - 1], X[N // 2, F // 2] = float("nan"), float("inf"), -float("inf")
+    out = hdc.levelid_encode(X, m)
+    ids, lo, hi, flip = (t.cpu().numpy() for t in hvs)
+    ref, _ = orc.levelid_encode(X.cpu().numpy(), ids, lo, hi, flip, L, -2.0, 2.5, np.arange(D))
+    assert np.array_equal(unpack(out.cpu().numpy().view(np.uint32), D), ref)
+
+
 def test_level_rows_that_switch_twice(hdc):
     """A level table of the caller's own: the slice with such a dim takes the other kernel."""
     F, D, L, N = 250, 3000, 16, 10100
