@@ -133,14 +133,13 @@ cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensor
 // Form of a call.  Two 128-row tiles a unit halve the class bytes streamed per
 // row (R x D bytes a unit); one tile a unit fills the chip with half the rows
 // and is the only form past 128 class rows (two D2 of 256 columns do not fit).
-// The estimate weighs a 256-dim tile of two at 5 and of one at 3.  Measured,
-// replays of one call with the workspace, the two-CTA form before (one tile a
-// unit, its class tile copied inside the expand -> MMA chain, bit-transposing
-// expansion) -> this one:
-//   10^5 x 16,384 dims: 100 classes 226.5 -> 194.2 us, 256 classes 393 -> 279
-//   10^6 x 1,024 dims:  100 classes 206.6 -> 153.2 us, 33 classes 168 -> 115
-// and without the workspace (classes expanded per tile) 365 -> 258 us at 10^5
-// x 16,384 x 100.
+// The estimate weighs a 256-dim tile of two at 5 and of one at 3.  Measured, calls
+// with the workspace, the two-CTA form before (one tile a unit, its class tile
+// copied inside the expand -> MMA chain, bit-transposing expansion, MMAs issued
+// under a lane test) -> this one:
+//   10^5 x 16,384 dims: 100 classes 234 -> 136 us, 256 classes 396 -> 240
+//   10^6 x 1,024 dims:  64 classes 185 -> 84 us, 200 classes 447 -> 234
+// and without it (classes expanded per tile) 365 -> 201 us at 10^5 x 16,384.
 cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *cls, int C, int W, int64_t D,
                                   int64_t s0, int64_t e0, int64_t stride, int32_t *labels, int32_t *dists,
                                   cudaStream_t st, uint8_t *signs)
