@@ -397,8 +397,9 @@ __device__ __forceinline__ void fence_to_async_global() { asm volatile("fence.pr
 // the MMA issuer frees it (a_free) once the last stage that reads it has
 // landed.
 // Work units: every role walks the same units, a query tile and a range of
-// its dim tiles (the whole tile unless p.nsplit > 1, a classify of fewer
-// tiles than SMs).  A split range's epilogue warps add their partial
+// its dim tiles (the whole tile unless p.nsplit > 1: a classify of fewer
+// tiles than SMs, or an encode whose ranges fill the last wave).  A split
+// classify range's epilogue warps add their partial
 // distances into p.dacc and count themselves in p.tile_done; the warp whose
 // count completes the tile reads the totals and takes the arg-min.
 // EWG = 2 or 4 (classify only): the epilogue warpgroups read the same TMEM
@@ -455,7 +456,7 @@ __global__ void __launch_bounds__(num_threads(EWG, QIN), 1)
     constexpr int KELEMS = ENC == HDC_ENC_BF16 ? BKB / 2 : BKB;
     // work units: (query tile, range of its dim tiles); one range per tile
     // unless the tile's dim tiles are split over several CTAs (nsplit)
-    const int NS = (CLASSIFY && !QIN) ? p.nsplit : 1;
+    const int NS = !QIN ? p.nsplit : 1;
     const int ntps = (num_n_tiles + NS - 1) / NS;   // dim tiles per range
     const int64_t num_units = num_m_tiles * NS;
 
