@@ -502,7 +502,7 @@ hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m, int32_t *
     fused.labels = labels; fused.dists = dists; fused.sims = scores;
     fused.cls_sign = m->cls_sign; fused.ldcs = m->ldcs;
     fused.dacc = (int32_t *)((char *)ws + L.dacc);
-    const bool fuse = use_tc(m) && !float_query(m->flags) && tc_supported(fused);
+    const bool fuse = use_tc(m) && !float_query(m->flags) && tc_supported(fused) && !tc_split_hamming(fused);
     const void *Xop;
     int64_t ldx;
     const float *sx;

@@ -190,6 +190,9 @@ bool tc_supported(const TcArgs &a);
 // split), and the words of a.dacc such a launch needs zeroed.
 int tc_split(const TcArgs &a);
 int64_t tc_split_words(const TcArgs &a);
+// Whether a classify of 33..112 binary classes encodes first, its tiles split over
+// the SMs, and then takes the packed Hamming kernel.
+bool tc_split_hamming(const TcArgs &a);
 // Whether the fused classify of a can quantise its own query tiles from the
 // FP32 rows a.X (binary classes: up to 32, or up to 112 with their E4M3
 // signs; 16-byte aligned rows of F % 4 == 0 floats; ldx <= 1024; at least two

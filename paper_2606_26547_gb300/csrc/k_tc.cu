@@ -206,6 +206,20 @@ int tc_split_encode(const TcArgs &a, int sms)
     return best;
 }
 
+// The fused kernel of 33..112 binary classes keeps whole query tiles, a tile's
+// stages one after another on one SM.  Up to half as many tiles as SMs the split
+// encode and the packed Hamming take less, from 24 stages a tile on (us, fused ->
+// split: 1 row of 1,024 x 8,192 x 112 124 -> 36, 9,728 rows 138 -> 88; 617 x 2,933
+// x 33, BF16 61 -> 26 and 68 -> 48; 617 x 1,024 x 100, 30 stages, 24 -> 22 and 37 ->
+// 31; 128 x 1,024 x 50, 6 stages, 9,728 rows 21 / 25).
+bool tc_split_hamming(const TcArgs &a)
+{
+    const int64_t m_tiles = (a.N + tc::BM - 1) / tc::BM;
+    const int kb = (a.ldx * (a.enc == HDC_ENC_BF16 ? 2 : 1) + tc::BKB - 1) / tc::BKB;
+    return a.nb == 1 && a.cls_sign && a.C > 32 && a.C <= tc::H_CMAX && m_tiles * 2 <= sm_count() &&
+           (a.Dk + tc::HBN - 1) / tc::HBN * kb >= 24 && hamming_packed_ok(a.C, a.W);
+}
+
 int64_t tc_split_words(const TcArgs &a) { return tc_split(a) > 1 ? a.N * a.C + (a.N + tc::BM - 1) / tc::BM : 0; }
 
 cudaError_t launch_tc_encode(const TcArgs &a, cudaStream_t st)
