@@ -274,7 +274,9 @@ cudaError_t tc_aux_read_status(cudaStream_t st, int *status);
 // runs (programmatic stream serialisation): early_wait returns when that kernel
 // is complete and its writes are visible, and lets the next launch start in
 // turn.  The pointers to what earlier kernels write pass through it: reads
-// through a const pointer are not ordered by the wait alone.
+// through a const pointer are not ordered by the wait alone.  Nor are __ldg
+// and other non-coherent loads, for data that does not change while the kernel
+// runs: these kernels run while the one before them still writes.
 template <typename P>
 __device__ __forceinline__ int read_after(P &p)
 {

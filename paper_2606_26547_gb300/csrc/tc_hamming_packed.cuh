@@ -552,12 +552,12 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
         // [2 * part, 2 * part + 2) with MT = 2 (2 R items), rows c0 and
         // c0 + 128 whole with MT = 1
         const int c0 = MT == 2 ? urow % p.R : urow, part = MT == 2 ? urow / p.R : 0;
-        auto class_words = [&](int c, int t) {
+        auto class_words = [&](int c, int t) {   // ordinary loads: an earlier kernel may write cls until grid_wait
             const bool ok = part < 2 && c < p.C && t * 4 < p.W;
             const uint32_t *w = p.cls + (int64_t)(ok ? c : 0) * p.W + (ok ? t * 4 : 0);
             if (!ok) return make_uint4(0, 0, 0, 0);
-            if (MT == 1) return __ldg(reinterpret_cast<const uint4 *>(w));
-            const uint2 h = __ldg(reinterpret_cast<const uint2 *>(w + part * 2));
+            if (MT == 1) return *reinterpret_cast<const uint4 *>(w);
+            const uint2 h = *reinterpret_cast<const uint2 *>(w + part * 2);
             return make_uint4(h.x, h.y, 0, 0);
         };
         const int tu0 = ch0 * 2 * HP_CHUNK, tun = min(ch1 * 2 * HP_CHUNK, 2 * p.nt) - tu0;   // a unit's atoms
