@@ -12,6 +12,7 @@
 namespace hdc {
 
 constexpr int kAlign = 256;  // alignment of every sub-buffer we carve
+constexpr size_t kMaxSmem = 227 * 1024;  // shared memory a block may have
 
 // Training groups samples with int32 offsets over up to 2N entries (a
 // retraining epoch places a misclassified sample in two groups) and 2C groups.
@@ -290,6 +291,17 @@ __device__ __forceinline__ void early_wait(P &...p)
     asm volatile("griddepcontrol.wait;" ::: "memory");
     (void)std::initializer_list<int>{read_after(p)...};
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
+// Lets kernel k be launched with up to `most` bytes of dynamic shared memory.  The
+// limit is the process's, one per kernel and device, and a smaller value lowers
+// it: callers pass the same constant for every call of a kernel, never the size
+// at hand, or a call of another host thread could lower the limit between this
+// and the launch.
+template <typename... P>
+cudaError_t allow_smem(void (*k)(P...), size_t most)
+{
+    return cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)most);
 }
 
 template <typename... P, typename... A>

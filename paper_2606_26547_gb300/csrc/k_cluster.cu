@@ -47,6 +47,7 @@ constexpr int STEP_PLANES = 7;     // counts up to STEP_ROWS
 constexpr int STEP_MAXK = 64;
 constexpr int UPD_SLICES = 16;     // most warps of an update block, each a part of the runs
 constexpr int CHIP_SMS = 152;
+constexpr size_t STEP_SMEM = 200 * 1024;   // most shared memory of an assignment block
 
 // Lines of the route, from both sides timed (us an iteration, 2 / 7 launches): a
 // block's planes are K W words a plane, so runs * K * W bounds the traffic
@@ -83,7 +84,7 @@ StepPlan step_plan(int64_t N, int W, int K)
     // an update block of 16 warps while the chip holds them all at once
     const int64_t blocks = (int64_t)W / 4 * K;
     for (p.slices = UPD_SLICES; p.slices > 2 && blocks * p.slices > CHIP_SMS * 48; p.slices /= 2) {}
-    p.ok = p.smem <= 200 * 1024;
+    p.ok = p.smem <= STEP_SMEM;
     return p;
 }
 
@@ -335,7 +336,7 @@ cudaError_t launch_step(const StepPlan &p, const uint32_t *H, int64_t N, int W, 
 {
     auto k = p.S == 4 ? assign_count_of<4>(p.cm) : assign_count_of<8>(p.cm);
     cudaError_t e = cudaSuccess;
-    if (first && p.smem > 40 * 1024) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)p.smem);
+    if (first) e = allow_smem(k, STEP_SMEM);
     if (e != cudaSuccess) return e;
     e = launch_early(k, dim3((unsigned)p.runs), (unsigned)(STEP_ROWS * p.S), p.smem, st, !first, H, N, W, K, p.chunks, p.rows,
                      p.words, p.runs, cls, mask ? 1 : 0, mask ? mask->s0 : 0, mask ? mask->e0 : 0, mask ? mask->stride : 1,

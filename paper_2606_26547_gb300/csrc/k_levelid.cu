@@ -651,6 +651,7 @@ LevelLayout level_layout(int F, int L, int Wk)
 }
 
 constexpr int SMS = 152;
+constexpr size_t FEW_SMEM = 220 * 1024, ENCODE_SMEM = 200 * 1024;   // most shared memory of a block; of staged rows
 
 template <int NFW>
 cudaError_t launch_count(const float *X, int64_t N, const hdc_levelid_model &m, uint32_t *H, int64_t slices, cudaStream_t st)
@@ -692,7 +693,7 @@ extern "C" hdc_status hdc_levelid_model_bytes(int32_t F, int32_t D, int32_t L, c
     if (!bytes || F <= 0 || D <= 0 || L < 2 || (cfg && cfg->struct_size < sizeof(hdc_approx_config)) ||
         !perf_of(D, cfg, &p))
         return HDC_ERR_INVALID_ARG;
-    if (F >= 8 * 1024 || encode_smem(F, L) > 200 * 1024) return HDC_ERR_UNSUPPORTED;
+    if (F >= 8 * 1024 || encode_smem(F, L) > ENCODE_SMEM) return HDC_ERR_UNSUPPORTED;
     *bytes = level_layout(F, L, words_for(p.Dk)).total;
     return HDC_OK;
 }
@@ -745,7 +746,7 @@ extern "C" hdc_status hdc_levelid_encode(const float *X, int64_t N, const hdc_le
                                          hdc_stream_t stream)
 {
     if (N < 0 || !m || m->struct_size < sizeof(hdc_levelid_model) || m->F <= 0 || m->L < 2 || m->Dk <= 0 ||
-        m->W != words_for(m->Dk) || !m->id || !m->level || encode_smem(m->F, m->L) > 200 * 1024 || m->F >= 8 * 1024)
+        m->W != words_for(m->Dk) || !m->id || !m->level || encode_smem(m->F, m->L) > ENCODE_SMEM || m->F >= 8 * 1024)
         return HDC_ERR_INVALID_ARG;
     if (N == 0) return HDC_OK;
     if (!X || !H) return HDC_ERR_INVALID_ARG;
@@ -763,11 +764,10 @@ extern "C" hdc_status hdc_levelid_encode(const float *X, int64_t N, const hdc_le
     for (int q1 = 1; q1 <= 4 && !many; q1 += 3) {
         const int64_t blocks = (N + LWARPS * q1 - 1) / (LWARPS * q1);
         const size_t smem = encode_smem(m->F, m->L) + (size_t)LWARPS * q1 * ((m->F + 3) / 4 * 4) * 4;
-        if (blocks * slices > SMS || smem > 220 * 1024 || (((uintptr_t)m->id | (uintptr_t)m->level) & 15)) continue;
+        if (blocks * slices > SMS || smem > FEW_SMEM || (((uintptr_t)m->id | (uintptr_t)m->level) & 15)) continue;
         auto k = hp_for(m->F) == 6 ? (q1 == 1 ? levelid_few_kernel<6, 1> : levelid_few_kernel<6, 4>)
                                    : (q1 == 1 ? levelid_few_kernel<9, 1> : levelid_few_kernel<9, 4>);
-        if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-            return HDC_ERR_CUDA;
+        if (allow_smem(k, FEW_SMEM) != cudaSuccess) return HDC_ERR_CUDA;
         k<<<dim3((unsigned)blocks, (unsigned)slices), LWARPS * 32, smem, st>>>(X, N, m->F, m->L, m->W, m->lo, m->scale, m->id,
                                                                               m->level, H);
         return cudaGetLastError() == cudaSuccess ? HDC_OK : HDC_ERR_CUDA;
@@ -777,8 +777,7 @@ extern "C" hdc_status hdc_levelid_encode(const float *X, int64_t N, const hdc_le
     auto k = hp_for(m->F) != 6 ? levelid_encode_kernel<9, false>
              : many            ? levelid_encode_kernel<6, true>
                                : levelid_encode_kernel<6, false>;
-    if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-        return HDC_ERR_CUDA;
+    if (allow_smem(k, ENCODE_SMEM + LOFF_BYTES) != cudaSuccess) return HDC_ERR_CUDA;
     // after the kernel above only what it left out: two blocks an SM, if any stay
     const int64_t blocks = (N + LQ - 1) / LQ;
     const dim3 grid((unsigned)(many ? std::min<int64_t>(blocks, (2 * SMS + slices - 1) / slices) : blocks), (unsigned)slices);

@@ -134,6 +134,7 @@ __global__ void __launch_bounds__(256) quant_rows_kernel(const float *__restrict
 // row maximum and converts straight from shared memory.  Waits are bounded
 // by the global timer; on expiry the kernel records status 1 and stops.
 constexpr int QSLOTS = 4, QWARPS = 4;
+constexpr size_t QSMEM_MAX = 200 * 1024;   // most shared memory of a block
 constexpr unsigned long long QTIMEOUT_NS = 2000000000ull;
 
 static __device__ int g_quant_status;
@@ -455,7 +456,7 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
     }
     const bool aligned_rows = F % 4 == 0 && lds % 4 == 0 && ((uintptr_t)src % 16) == 0;
     const size_t qsmem = (size_t)QWARPS * QSLOTS * F * 4 + (size_t)QWARPS * QSLOTS * 8;
-    if (aligned_rows && qsmem <= 200 * 1024) {
+    if (aligned_rows && qsmem <= QSMEM_MAX) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -466,8 +467,7 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
         if (!zero.early) qblocks = (int64_t)sms * per_sm;
 #define HDC_QBULK(E)                                                                                              \
     do {                                                                                                          \
-        cudaError_t e = cudaFuncSetAttribute(quant_rows_bulk_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                             (int)qsmem);                                                         \
+        cudaError_t e = allow_smem(quant_rows_bulk_kernel<E>, QSMEM_MAX);                                         \
         if (e != cudaSuccess) return e;                                                                           \
         quant_rows_bulk_kernel<E><<<(unsigned)qblocks, QWARPS * 32, qsmem, st>>>(src, lds, row_off, row_step,     \
                                                                                  nrows, F, dst, ldd, scale, zero); \
@@ -482,7 +482,7 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
     }
     // rows not 16-byte aligned: their aligned spans streamed the same way
     const size_t ssmem = (size_t)QWARPS * QSLOTS * span_slot_bytes(F) + (size_t)QWARPS * QSLOTS * 8;
-    if (ssmem <= 200 * 1024 && ldd % 4 == 0) {
+    if (ssmem <= QSMEM_MAX && ldd % 4 == 0) {
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -493,8 +493,7 @@ cudaError_t launch_quant_rows(const float *src, int64_t lds, int64_t row_off, in
         if (!zero.early) qblocks = (int64_t)sms * per_sm;
 #define HDC_QSPAN(E)                                                                                              \
     do {                                                                                                          \
-        cudaError_t e = cudaFuncSetAttribute(quant_rows_span_kernel<E>, cudaFuncAttributeMaxDynamicSharedMemorySize, \
-                                             (int)ssmem);                                                         \
+        cudaError_t e = allow_smem(quant_rows_span_kernel<E>, QSMEM_MAX);                                         \
         if (e != cudaSuccess) return e;                                                                           \
         quant_rows_span_kernel<E><<<(unsigned)qblocks, QWARPS * 32, ssmem, st>>>(src, lds, row_off, row_step,     \
                                                                                  nrows, F, dst, ldd, scale, zero); \

@@ -373,10 +373,7 @@ cudaError_t launch_csa_cm(const uint32_t *Q, int64_t N, const uint32_t *cls, int
     const int WC = w16 < 512 ? w16 : 512;
     const size_t smem = ((size_t)QRING * TPB * 4 + (size_t)CM * WC + (MASKED ? WC : 0)) * sizeof(uint32_t);
     auto k = hamming_csa_kernel<CM, MASKED, HIST>;
-    if (smem > 48 * 1024) {
-        cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return e;
-    }
+    static_assert((QRING * TPB * 4 + CM * 512 + 512 + 2 * CM) * sizeof(uint32_t) <= 48 * 1024, "shared memory without opt-in");
     const int64_t blocks = (N + TPB / 4 - 1) / (TPB / 4);
     k<<<(unsigned)blocks, TPB, smem, st>>>(Q, N, cls, C, W, WC, s0, e0, stride, labels, dists, y, hist);
     return cudaGetLastError();
@@ -441,8 +438,9 @@ cudaError_t launch_nb(const uint32_t *Q, int64_t N, const uint32_t *planes, int 
     if (WCH > 256) WCH = 256;
     if (WCH > W) WCH = W;
     const size_t smem = ((size_t)C * TPB + (size_t)NB * C * WCH + WCH) * sizeof(uint32_t);
-    if (smem > 200 * 1024) return cudaErrorNotSupported;
-    cudaError_t e = cudaFuncSetAttribute(similarity_kernel<NB>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr size_t most = 200 * 1024;
+    if (smem > most) return cudaErrorNotSupported;
+    cudaError_t e = allow_smem(similarity_kernel<NB>, most);
     if (e != cudaSuccess) return e;
     const int use_mask = p != nullptr;
     const int64_t s0 = p ? p->s0 : 0, e0 = p ? p->e0 : D, stride = p ? p->stride : 1;

@@ -440,6 +440,8 @@ bool make_conf(const hdc_sweep_spec *sp, int64_t D, SweepConf *cf)
     return true;
 }
 
+constexpr size_t kSweepSmem = 220 * 1024;   // most shared memory of a popcount block
+
 struct SweepLayout {
     size_t planes, sums, norms, total;   // tensor-core route: digit rows, sums of squares
 };
@@ -498,7 +500,7 @@ extern "C" hdc_status hdc_sweep_eval(const uint32_t *H, const int32_t *y, int64_
     int maxp = 0;
     for (int j = 0; j < cf.nb; j++) maxp = cf.planes[j] > maxp ? cf.planes[j] : maxp;
     const size_t smem = (size_t)cf.ns * C * tpb * 8 + (size_t)wch * (tpb + 1) * 4 + (size_t)maxp * C * wch * 4;
-    if (smem > 220 * 1024) return HDC_ERR_UNSUPPORTED;
+    if (smem > kSweepSmem) return HDC_ERR_UNSUPPORTED;
     cudaStream_t st = (cudaStream_t)stream;
     char *w = (char *)ws;
     if (cudaMemsetAsync(correct, 0, ncfg * sizeof(int32_t), st) != cudaSuccess) return HDC_ERR_CUDA;
@@ -538,9 +540,7 @@ extern "C" hdc_status hdc_sweep_eval(const uint32_t *H, const int32_t *y, int64_
                                          (double *)(w + L.norms));
     if (cudaGetLastError() != cudaSuccess) return HDC_ERR_CUDA;
     if (N == 0) return HDC_OK;
-    if (cudaFuncSetAttribute(sweep_eval_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-        return HDC_ERR_CUDA;
+    if (allow_smem(sweep_eval_kernel, kSweepSmem) != cudaSuccess) return HDC_ERR_CUDA;
     const int64_t blocks = (N + tpb - 1) / tpb;
     sweep_eval_kernel<<<dim3((unsigned)blocks, (unsigned)cf.nb), tpb, smem, st>>>(H, y, N, C, W, wch, cf, (const uint32_t *)(w + L.planes),
                                                           (const long long *)(w + L.sums),

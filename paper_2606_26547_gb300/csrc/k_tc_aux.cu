@@ -103,13 +103,13 @@ cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensor
     // shared memory: the query ring, the class atoms, barriers; at least 120 KB
     // so that no second CTA shares the SM and waits for its TMEM columns
     const size_t fixed = 1024 + tc::hp_q_bytes(pl.mt) + tc::hp_tail(pl.mt), atom = (size_t)p.R * 128;
-    size_t nbs = (227 * 1024 - fixed) / atom;
+    size_t nbs = (kMaxSmem - fixed) / atom;
     if (nbs > (size_t)tc::HP_NBS_MAX) nbs = tc::HP_NBS_MAX;
     p.nbs = (int)nbs;
     size_t smem = fixed + (PRE ? nbs * atom : tc::hp_nab(pl.mt, false) * atom + (size_t)((p.W + 3) & ~3) * 4);
     if (smem < 120 * 1024) smem = 120 * 1024;
     auto k = pl.mt == 2 ? tc::tc_hamming_packed_kernel<2, PRE, FIN> : tc::tc_hamming_packed_kernel<1, PRE, FIN>;
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, kMaxSmem);
     if (e != cudaSuccess) return e;
     const int64_t ctas = pl.units * pl.S;
     cudaLaunchConfig_t lc = {};

@@ -413,7 +413,7 @@ static cudaError_t launch_fcos_stages(const CUtensorMap &ma, const CUtensorMap &
 {
     auto k = tc_fcos_kernel<ENC, STAGES, B2BUF>;
     const size_t smem = fc_smem_bytes(STAGES, p.Cp, B2BUF);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, kMaxSmem);
     if (e != cudaSuccess) return e;
     return launch_after(k, grid, FC_THREADS, smem, st, ma, mb, mv, p);
 }

@@ -426,7 +426,7 @@ static cudaError_t launch_hamming_q(const CUtensorMap &ma, const CUtensorMap &mb
 {
     auto k = tc_hamming_kernel<ENC, QIN>;
     const size_t smem = h_smem_bytes(p.Cp);
-    cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = allow_smem(k, kMaxSmem);
     if (e != cudaSuccess) return e;
     return launch_after(k, grid, h_threads(QIN), smem, st, ma, mb, ms, p);
 }
