@@ -206,8 +206,6 @@ size_t tc_stage_bytes(const TcArgs &a);
 // Reads and clears the streaming quantiser's device status word.
 cudaError_t quant_read_status(cudaStream_t st, int *status);
 
-// Most rows of the tensor-core Hamming kernel (32-bit row coordinates).
-constexpr int64_t kMaxPackedRows = 0x7fffffffLL - 256;
 // Reads and clears the tensor-core kernels' device status word.
 cudaError_t tc_read_status(cudaStream_t st, int *status);
 // Hamming arg-min of packed rows on the tensor cores (up to 256 binary

@@ -468,7 +468,7 @@ cudaError_t launch_similarity(const uint32_t *Q, int64_t N, const uint32_t *plan
     // 100,000 x 16,384 dims x 32: 193 us, popcounts 428; 10,000 x 4,096 x 17:
     // 15.6 / 22.9; equal where a launch's latency is all (300 x 1,024).  Up to
     // 16 classes the carry-save kernel above is the faster (x 16: 160 / 191).
-    if (nb == 1 && hamming_packed_ok(C, W) && (C > 32 || N <= kMaxPackedRows))
+    if (nb == 1 && hamming_packed_ok(C, W))
         return launch_hamming_packed(Q, N, planes, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      dists, st);
     if (nb == 1 && C <= 32) return launch_reg<32>(Q, N, planes, C, W, D, p, labels, dists, st);

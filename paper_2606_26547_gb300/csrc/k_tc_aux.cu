@@ -91,7 +91,7 @@ HpPlan hp_plan(int64_t N, int mt, int chunks, int sms, int tile_cost)
 // Chooses the form of a task whose sizes and epilogue `p` holds, and launches
 // it: mq the packed rows, mc the class bytes (PRE).
 template <bool PRE, int FIN>
-cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensorMap &mc, cudaStream_t st)
+cudaError_t launch_packed_rows(tc::HPParams &p, const CUtensorMap &mq, const CUtensorMap &mc, cudaStream_t st)
 {
     const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
     HpPlan pl = hp_plan(p.N, 1, chunks, sms, 3);
@@ -128,6 +128,27 @@ cudaError_t launch_packed(tc::HPParams &p, const CUtensorMap &mq, const CUtensor
     lc.numAttrs = pl.S > 1 ? 2 : 1;
     return cudaLaunchKernelEx(&lc, k, p, mq, mc);
 }
+
+// The rows Q in launches whose row coordinates fit the copies' 32 bits, whole
+// 256-row units each.
+constexpr int64_t HP_LAUNCH_ROWS = 0x7fffff00;
+template <bool PRE, int FIN>
+cudaError_t launch_packed(const tc::HPParams &all, const uint32_t *Q, const CUtensorMap *mc, cudaStream_t st)
+{
+    cudaError_t e = cudaSuccess;
+    for (int64_t r0 = 0; r0 < all.N && e == cudaSuccess; r0 += HP_LAUNCH_ROWS) {
+        tc::HPParams p = all;
+        p.N = all.N - r0 < HP_LAUNCH_ROWS ? all.N - r0 : HP_LAUNCH_ROWS;
+        if (p.labels) p.labels += r0;
+        if (p.dists) p.dists += r0 * p.C;
+        if (p.scores) p.scores += r0 * p.C;
+        if (p.y) p.y += r0;
+        CUtensorMap mq;
+        if (!make_packed_map(&mq, Q + r0 * p.W, p.W, p.N)) return cudaErrorInvalidValue;
+        e = launch_packed_rows<PRE, FIN>(p, mq, mc ? *mc : mq, st);
+    }
+    return e;
+}
 }  // namespace
 
 // Form of a call.  Two 128-row tiles a unit halve the class bytes streamed per
@@ -145,11 +166,9 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
                                   cudaStream_t st, uint8_t *signs)
 {
     if (N <= 0) return cudaSuccess;
-    if (!hamming_packed_ok(C, W) || stride < 1 || N > kMaxPackedRows) return cudaErrorNotSupported;
+    if (!hamming_packed_ok(C, W) || stride < 1) return cudaErrorNotSupported;
     const int ldcs = hamming_packed_ldcs(W), R = (C + 15) / 16 * 16;
-    CUtensorMap mq, mc;
-    if (!make_packed_map(&mq, Q, W, N)) return cudaErrorInvalidValue;
-    mc = mq;
+    CUtensorMap mc;
     if (signs) {   // the classes once into `signs`, zero outside the kept dims
         const int64_t n = (int64_t)C * (ldcs / 4);
         class_bytes_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(cls, C, W, ldcs / 4, D, s0, e0, stride,
@@ -173,7 +192,7 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
     p.kept = end > s0 ? (int)((end - s0 + stride - 1) / stride) : 0;
     p.labels = labels;
     p.dists = dists;
-    return signs ? launch_packed<true, tc::HP_HAMMING>(p, mq, mc, st) : launch_packed<false, tc::HP_HAMMING>(p, mq, mc, st);
+    return signs ? launch_packed<true, tc::HP_HAMMING>(p, Q, &mc, st) : launch_packed<false, tc::HP_HAMMING>(p, Q, nullptr, st);
 }
 
 cudaError_t launch_packed_cosine(const uint32_t *Q, int64_t N, int W, const uint8_t *vals, int C, int P,
@@ -181,9 +200,9 @@ cudaError_t launch_packed_cosine(const uint32_t *Q, int64_t N, int W, const uint
 {
     if (N <= 0) return cudaSuccess;
     const int rows = C * P, R = (rows + 15) / 16 * 16, ld = hamming_packed_ldcs(W);
-    if (!hamming_packed_ok(rows, W) || P < 1 || P > 2 || N > 0x7fffffffLL - 2 * tc::BM) return cudaErrorNotSupported;
-    CUtensorMap mq, mc;
-    if (!make_packed_map(&mq, Q, W, N) || !make_class_sign_map(&mc, vals, ld, rows, R)) return cudaErrorInvalidValue;
+    if (!hamming_packed_ok(rows, W) || P < 1 || P > 2) return cudaErrorNotSupported;
+    CUtensorMap mc;
+    if (!make_class_sign_map(&mc, vals, ld, rows, R)) return cudaErrorInvalidValue;
     tc::HPParams p = {};
     p.N = N;
     p.W = W;
@@ -194,7 +213,7 @@ cudaError_t launch_packed_cosine(const uint32_t *Q, int64_t N, int W, const uint
     p.cnorm = cnorm;
     p.labels = labels;
     p.scores = scores;
-    return launch_packed<true, tc::HP_COSINE>(p, mq, mc, st);
+    return launch_packed<true, tc::HP_COSINE>(p, Q, &mc, st);
 }
 
 cudaError_t launch_packed_sweep(const PackedSweep &a, cudaStream_t st)
@@ -208,13 +227,10 @@ cudaError_t launch_packed_sweep(const PackedSweep &a, cudaStream_t st)
         p.cfg_col[i] = (uint16_t)rows;
         rows += a.C * (a.digits[i] ? a.digits[i] : 1);
     }
-    if (a.ncfg > tc::HP_MAXCFG || !hamming_packed_ok(rows, a.W) || a.N > 0x7fffffffLL - 2 * tc::BM)
-        return cudaErrorNotSupported;
+    if (a.ncfg > tc::HP_MAXCFG || !hamming_packed_ok(rows, a.W)) return cudaErrorNotSupported;
     const int R = (rows + 15) / 16 * 16;
-    CUtensorMap mq, mc;
-    if (!make_packed_map(&mq, a.H, a.W, a.N) ||
-        !make_class_sign_map(&mc, a.vals, hamming_packed_ldcs(a.W), rows, R))
-        return cudaErrorInvalidValue;
+    CUtensorMap mc;
+    if (!make_class_sign_map(&mc, a.vals, hamming_packed_ldcs(a.W), rows, R)) return cudaErrorInvalidValue;
     p.N = a.N;
     p.W = a.W;
     p.C = a.C;
@@ -225,7 +241,8 @@ cudaError_t launch_packed_sweep(const PackedSweep &a, cudaStream_t st)
     p.y = a.y;
     p.correct = a.correct;
     p.labels = a.labels;
-    return launch_packed<true, tc::HP_SWEEP>(p, mq, mc, st);
+    p.ldl = a.N;
+    return launch_packed<true, tc::HP_SWEEP>(p, a.H, &mc, st);
 }
 
 cudaError_t launch_wait_selftest(unsigned long long limit_ns, cudaStream_t st)

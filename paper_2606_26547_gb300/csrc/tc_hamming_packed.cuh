@@ -103,6 +103,7 @@ struct HPParams {
     int ncfg;
     uint8_t cfg_p[HP_MAXCFG], cfg_k[HP_MAXCFG];
     uint16_t cfg_col[HP_MAXCFG];
+    int64_t ldl;             // labels from one output entry to the next
     const long long *sumsq;
     const int32_t *y;
     int32_t *correct;
@@ -453,7 +454,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             } else {
                 best = arg_max(row, valid, col, f * p.C, nullptr, HpInt<8>(), cols8);
             }
-            if (valid && p.labels) p.labels[(int64_t)p.cfg_k[f] * p.N + row] = best;
+            if (valid && p.labels) p.labels[(int64_t)p.cfg_k[f] * p.ldl + row] = best;
             const unsigned hit = __ballot_sync(0xffffffffu, valid && best == yv);
             if (lane == 0 && hit) atomicAdd(p.correct + p.cfg_k[f], __popc(hit));
         }
