@@ -312,9 +312,14 @@ hdc_status hdc_classify_host(const float *const *parts_host, const int64_t *part
  *   bits[j]     1 (Hamming, arg-min), 4 or 8 (b-bit cosine, arg-max, as in
  *               hdc_classify), or 0: cosine against the unquantised int32
  *               accumulators themselves (requires sum over D of acc^2 < 2^63)
+ * Configurations of at most 256 class rows (C at 1 and 4 bits, 2 C at 8, 8 C
+ * at 0) of D <= 131072 dims are scored on the tensor cores, else by popcounts.
  * block_threads / words_per_chunk are launch-shape knobs (0 = default;
- * 64, 128 or 256 threads; a multiple of 4 words) chosen by an autotuner;
- * results do not depend on them.                                           */
+ * 64, 128 or 256 threads; a multiple of 4 words) of the popcount form, chosen
+ * by an autotuner; results do not depend on them.  HDC_ERR_UNSUPPORTED, on
+ * either form, when its shared memory would exceed 220 KB: with t threads and
+ * w words (128 and 32 by default, w at most W(D)) and P bits of the widest
+ * width (32 for 0), 8 n_strides C t + 4 w (t + 1) + 4 P C w bytes.          */
 #define HDC_SWEEP_MAX_STRIDES 6
 #define HDC_SWEEP_MAX_BITS 4
 typedef struct {

@@ -4,6 +4,10 @@ Times every candidate (threads per block, words per shared-memory chunk) of
 hdc_sweep_eval on the caller's own data with CUDA events, keeps the fastest
 and caches the choice per (device, shape) in a JSON file.  Results of the
 kernel do not depend on the launch shape, so tuning never changes output.
+
+Only the popcount form reads the launch shape.  Where the tensor-core form
+takes the sweep every candidate is the same launch: there is nothing to time,
+and the first one the library accepts is returned.
 """
 from __future__ import annotations
 
@@ -57,8 +61,22 @@ def pick_fastest(timings: dict):
     return best
 
 
+def tensor_core_sweep(D, C, bits) -> bool:
+    """Whether hdc_sweep_eval scores these widths on the tensor cores: rows of
+    up to 4,096 words, and at most 256 rows of base-16 digits a configuration."""
+    return hdc.words(D) <= 4096 and all(C * {0: 8, 8: 2}.get(b, 1) <= 256 for b in bits)
+
+
 def tune_sweep(H, y, acc, D, C, strides, bits, reps: int = 3, use_cache: bool = True):
     """(block_threads, words_per_chunk) for hdc_sweep_eval on this shape."""
+    if tensor_core_sweep(D, C, bits):
+        for bt, wc in CANDIDATES:
+            try:
+                hdc.Sweep(D, C, strides, bits, H.shape[0], H.device, bt, wc)(H, y, acc)
+                return bt, wc
+            except hdc.HdcError:
+                continue  # the popcount form's shared memory: refused on either form
+        return 0, 0
     key = sweep_key(H.shape[0], D, C, strides, bits)
     cache = _load() if use_cache else {}
     if key in cache:
