@@ -7,7 +7,7 @@
 // form of the method; with BF16/FP8 inputs the products are exact in FP32,
 // which gives a CUDA-core cross-check of the tensor-core encoder.
 //
-// Tiling: 128 queries x 64 * CG dims per block (CG = 4, or 2 where that leaves
+// Tiling: 128 queries x 64 * CG dims per block (CG = 4, or 2 with few features or where that leaves
 // SMs idle), K slabs of 16, 256 threads with 8 x 4 * CG outputs each (rows
 // ty*4+{0..3} and 64+ty*4+{0..3}, columns tx*4+{0..3} of every 64),
 // double-buffered shared memory with register prefetch.
@@ -232,9 +232,13 @@ cudaError_t launch_encode_simt(const void *X, int64_t ldx, int64_t N, int F, con
         // each at half the rate; a lone one at the full rate), in 128 x 128
         // tiles; the wide one runs ~10 % faster where both fill the chip
         // (5,000 x 617 x 2,048, 2.1 waves of the wide tile: 284 us narrow, 338 us wide).
+        // Not below 16 K slabs: a block's own ends, the stores of its projections
+        // above all, pass beside another block's multiply-adds on the narrow tile
+        // only (42,413 x 10 x 1,685 with projections: 136 us narrow, 177 wide; x 64:
+        // 252 / 302; without, x 16: 64 / 78; from 300 features 0.9 .. 1.04).
         const int64_t mt = (n + BM - 1) / BM, bw = mt * ((Dk + 255) / 256), bn = mt * ((Dk + 127) / 128);
         const int64_t rem = bn % 304, cn = bn / 304 * 2 + (rem > 152 ? 2 : rem > 0 ? 1 : 0);
-        const bool wide = (bw + 151) / 152 * 18 < cn * 10;
+        const bool wide = F >= 16 * BK && (bw + 151) / 152 * 18 < cn * 10;
         cudaError_t e;
 #define HDC_SIMT(T, V) \
     (wide ? launch_simt<T, V, 4>(Xc, ldx, n, F, Bq, ldb, Dk, sxc, sb, Hc, W, sc, st) \
