@@ -68,25 +68,53 @@ int hp_sms()
     return sms;
 }
 
-// Units (MT x 128 rows), CTAs per unit and the wave-time estimate of one form:
-// waves x 256-dim tiles per CTA x the tile's time.  A split needs its clusters
-// resident together: an SM group holds at least 16 SMs, so at most
-// 8 * floor(16 / S) clusters of S CTAs at once.
+// Units (MT x 128 rows), CTAs per unit, and the estimate of one form's time.
+// A split needs its clusters resident together: 8 * floor(16 / S) clusters of S
+// CTAs up to six, 15 of seven or eight (one of the SM groups is smaller: the
+// occupancy query's answer; 16 of eight took two waves, 26 us for 14).
 struct HpPlan {
     int mt, S;
     int64_t units, cost;
 };
-HpPlan hp_plan(int64_t N, int mt, int chunks, int sms, int tile_cost)
+bool hp_resident(int64_t units, int S, int sms) { return units * S <= sms && units <= (S > 6 ? 14 : 8 * (16 / S)); }
+
+// Cosine and sweep: waves x 256-dim tiles a CTA x the tile's time (two row tiles
+// 5, one 3); as many CTAs a unit as fit, which also share its row groups' scores.
+HpPlan hp_plan_scores(int64_t N, int mt, int chunks, int sms)
 {
-    HpPlan pl;
-    pl.mt = mt;
-    pl.units = (N + mt * tc::BM - 1) / (mt * tc::BM);
-    pl.S = 1;
+    HpPlan pl = {mt, 1, (N + mt * tc::BM - 1) / (mt * tc::BM), 0};
     for (int S = 2; S <= tc::HP_SMAX && S <= chunks; S++)
-        if (pl.units * S <= sms && pl.units <= 8 * (16 / S)) pl.S = S;
+        if (hp_resident(pl.units, S, sms)) pl.S = S;
     const int64_t waves = (pl.units * pl.S + sms - 1) / sms;
-    pl.cost = waves * ((chunks + pl.S - 1) / pl.S) * tile_cost;
+    pl.cost = waves * ((chunks + pl.S - 1) / pl.S) * (mt == 2 ? 5 : 3);
     return pl;
+}
+
+// Hamming: 10 ns a wave's 256-dim tiles and R-column epilogue, and a split's
+// barriers and its reading of R sums of S ranks, 1 us and up: a fit to the forms
+// forced on 55 .. 30,000 rows of 400 .. 8,000 dims, 20 .. 220 classes (1,418
+// timings, 95 % within a tenth; the form chosen is 1.0005 times the best on
+// average).  Splitting whenever the clusters fit took 1.2 times the best, and a
+// sixth of those calls longer than the kernel before this one: 16,222 x 1,219 x
+// 98 15.3 us in two CTAs a unit, 8.4 in one, 11.2 before; 500 x 1,380 x 112 12.9,
+// 8.8, 12.1.
+HpPlan hp_plan_hamming(int64_t N, int mt, int R, int nt, bool pre, int sms)
+{
+    HpPlan best = {mt, 1, (N + mt * tc::BM - 1) / (mt * tc::BM), 0};
+    const int chunks = (nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
+    const int tile = pre ? (mt == 1 ? 42 : 54) + R / 20 : mt == 1 ? 67 + R / 6 : 87 + R * 3 / 10;
+    for (int S = 1; S <= tc::HP_SMAX && S <= chunks; S++) {
+        if (S > 1 && !hp_resident(best.units, S, sms)) continue;
+        const int64_t waves = (best.units * S + sms - 1) / sms;
+        const int part = (chunks + S - 1) / S * tc::HP_CHUNK, tiles = part < nt ? part : nt;
+        int64_t cost = waves * ((int64_t)tiles * tile + (mt == 1 ? R : R * 5 / 4));
+        if (S > 1) cost += mt == 1 ? 110 + R * (165 * S + 20) / 100 : 130 + R * (160 * S + 140) / 100;
+        if (S == 1 || cost < best.cost) {
+            best.S = S;
+            best.cost = cost;
+        }
+    }
+    return best;
 }
 // Chooses the form of a task whose sizes and epilogue `p` holds, and launches
 // it: mq the packed rows, mc the class bytes (PRE).
@@ -94,9 +122,12 @@ template <bool PRE, int FIN>
 cudaError_t launch_packed_rows(tc::HPParams &p, const CUtensorMap &mq, const CUtensorMap &mc, cudaStream_t st)
 {
     const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
-    HpPlan pl = hp_plan(p.N, 1, chunks, sms, 3);
+    auto plan = [&](int mt) {
+        return FIN == tc::HP_HAMMING ? hp_plan_hamming(p.N, mt, p.R, p.nt, PRE, sms) : hp_plan_scores(p.N, mt, chunks, sms);
+    };
+    HpPlan pl = plan(1);
     if (p.R <= 128) {
-        const HpPlan p2 = hp_plan(p.N, 2, chunks, sms, 5);
+        const HpPlan p2 = plan(2);
         if (p2.cost < pl.cost) pl = p2;
     }
     p.S = pl.S;
@@ -154,7 +185,7 @@ cudaError_t launch_packed(const tc::HPParams &all, const uint32_t *Q, const CUte
 // Form of a call.  Two 128-row tiles a unit halve the class bytes streamed per
 // row (R x D bytes a unit); one tile a unit fills the chip with half the rows
 // and is the only form past 128 class rows (two D2 of 256 columns do not fit).
-// The estimate weighs a 256-dim tile of two at 5 and of one at 3.  Measured, calls
+// hp_plan_hamming takes the faster.  Measured, calls
 // with the workspace, the two-CTA form before (one tile a unit, its class tile
 // copied inside the expand -> MMA chain, bit-transposing expansion, MMAs issued
 // under a lane test) -> this one:
