@@ -118,6 +118,17 @@ struct TrainScratch {
 // clustering workspaces (0 outside 17..256).
 size_t class_sign_bytes(int C, int W);
 size_t scratch_sign_bytes(int C, int W);
+// Whether 17..32 classes are compared by popcounts all the same: small calls of
+// narrow rows, where the packed kernel's set-up and 1,024-dim query chunks are
+// all of its time (us, popcounts / packed, the same for 17 and 32 classes: 1,000 x
+// 900 5.3 / 7.1, x 2,048 8.8 / 9.6, x 3,000 12.2 / 9.9; 10,000 x 900 6.8 / 7.2, x
+// 1,200 9.0 / 8.2; 19,456 x 256 4.9 / 5.1, x 500 6.0 / 5.9; 60,000 x 100 8.2 /
+// 7.2).  With the classes to be expanded first (`scratch`) up to 1,024 dims: a
+// retraining epoch of 1,000 rows x 900 16.4 / 18.5, x 1,200 and x 2,048 equal.
+inline bool few_classes_popcount(int64_t N, int C, int W, bool scratch)
+{
+    return C <= 32 && W <= (scratch ? 32 : 64) && N * W <= 260000;
+}
 // Hamming arg-min of N packed rows against C classes over the kept dims
 // (s0, s0 + stride, ... < e0; all of [0, D) for a stride-1 full range): the
 // library's routes, with the class hypervectors expanded into `signs`

@@ -466,9 +466,9 @@ cudaError_t launch_similarity(const uint32_t *Q, int64_t N, const uint32_t *plan
     // rows expanded to +-1, whose time hardly depends on the classes where the
     // popcount loop is bound by the popcount unit (~16 per clock per SM).
     // 100,000 x 16,384 dims x 32: 193 us, popcounts 428; 10,000 x 4,096 x 17:
-    // 15.6 / 22.9; equal where a launch's latency is all (300 x 1,024).  Up to
-    // 16 classes the carry-save kernel above is the faster (x 16: 160 / 191).
-    if (nb == 1 && hamming_packed_ok(C, W))
+    // 15.6 / 22.9; the other way round in small calls (few_classes_popcount).  Up to
+    // 16 classes the carry-save kernel above is the faster (x 16: 142 / 191).
+    if (nb == 1 && hamming_packed_ok(C, W) && !few_classes_popcount(N, C, W, false))
         return launch_hamming_packed(Q, N, planes, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      dists, st);
     if (nb == 1 && C <= 32) return launch_reg<32>(Q, N, planes, C, W, D, p, labels, dists, st);

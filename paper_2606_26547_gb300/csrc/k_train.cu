@@ -546,7 +546,7 @@ cudaError_t launch_argmin_ws(const uint32_t *H, int64_t N, const uint32_t *cls, 
                              const Perf *p, int32_t *labels, uint8_t *signs, cudaStream_t st)
 {
     if (N <= 0) return cudaSuccess;
-    if (signs && scratch_sign_bytes(C, W) > 0) {
+    if (signs && scratch_sign_bytes(C, W) > 0 && !few_classes_popcount(N, C, W, true)) {
         // expand the classes once, then stream them to the tensor-core route
         return launch_hamming_packed(H, N, cls, C, W, D, p ? p->s0 : 0, p ? p->e0 : D, p ? p->stride : 1, labels,
                                      nullptr, st, signs);
