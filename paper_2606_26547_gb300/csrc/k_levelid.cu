@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(LWARPS * 32) levelid_encode_kernel(const float
 // where there are four queries.  Here the rows are staged by asynchronous
 // copies while all of the queries' levels are formed, and a warp takes Q1
 // queries: one while the blocks fit the SMs, four then.  One query, 561 x 4,928,
-// 128 levels 48 -> 15 us; 1,000, 617 x 1,024 62 -> 19 (four a warp, 3,000: 64 -> 54).
+// 128 levels 48 -> 11 us; 1,000, 617 x 1,024 62 -> 15 (four a warp, 3,000: 64 -> 41).
 template <int HP, int Q1>
 __global__ void __launch_bounds__(LWARPS * 32) levelid_few_kernel(const float *__restrict__ X, int64_t N, int F, int L, int W,
                                                                 float lo, float scale, const uint32_t *__restrict__ id,
@@ -271,11 +271,24 @@ __global__ void __launch_bounds__(LWARPS * 32) levelid_few_kernel(const float *_
     asm volatile("cp.async.commit_group;");
     const int64_t q0 = ((int64_t)blockIdx.x * LWARPS + warp) * Q1;   // this warp's queries
     int *off = soff + warp * Q1 * Fp;
+    // a step's loads all in flight, the partial one's too: left to the loop's
+    // remainder they waited for memory up to three times more a query, so that
+    // F = 225 .. 255 took longer than the kernel above (3,000 x 232 x 500: 28.1 us,
+    // 23.9 there; 17.0 so)
+    constexpr int FU = Q1 == 1 ? 8 : 4;
+    for (int f0 = lane; f0 < F; f0 += 32 * FU) {
+        float x[Q1][FU];
 #pragma unroll
-    for (int a = 0; a < Q1; a++)
-#pragma unroll 8
-        for (int f = lane; f < F; f += 32)
-            off[a * Fp + f] = q0 + a < N ? quant_level(__ldg(X + (q0 + a) * F + f), lo, scale, L) * LWC : 0;
+        for (int a = 0; a < Q1; a++)
+#pragma unroll
+            for (int u = 0; u < FU; u++)
+                x[a][u] = f0 + 32 * u < F && q0 + a < N ? __ldg(X + (q0 + a) * F + f0 + 32 * u) : 0.f;
+#pragma unroll
+        for (int a = 0; a < Q1; a++)
+#pragma unroll
+            for (int u = 0; u < FU; u++)   // rows past N: not stored
+                if (f0 + 32 * u < F) off[a * Fp + f0 + 32 * u] = quant_level(x[a][u], lo, scale, L) * LWC;
+    }
     asm volatile("cp.async.wait_group 0;" ::: "memory");
     __syncthreads();
     if (q0 >= N) return;
