@@ -207,17 +207,24 @@ int tc_split_encode(const TcArgs &a, int sms)
 }
 
 // The fused kernel of 33..112 binary classes keeps whole query tiles, a tile's
-// stages one after another on one SM.  Up to half as many tiles as SMs the split
-// encode and the packed Hamming take less, from 24 stages a tile on (us, fused ->
-// split: 1 row of 1,024 x 8,192 x 112 124 -> 36, 9,728 rows 138 -> 88; 617 x 2,933
-// x 33, BF16 61 -> 26 and 68 -> 48; 617 x 1,024 x 100, 30 stages, 24 -> 22 and 37 ->
-// 31; 128 x 1,024 x 50, 6 stages, 9,728 rows 21 / 25).
+// stages one after another on one SM.  The split encode and the packed Hamming
+// spread them, for two launches more and a read of the packed rows.  The line is a
+// fit to both sides at 128 .. 1,000 features, 400 .. 8,000 dims, 33 .. 111 classes
+// and 1 .. 9,728 rows (1,230 points; the side taken is 1.003 times the faster on
+// average): what is spread counts less as the tiles fill the SMs by themselves,
+// the dim tiles' own time not at all at half of them.  us on the device, fused /
+// split, 111 classes:
+//   one row    617 x 800, 25 stages 15.2 / 17.5; x 1,024, BF16, 60 stages 22.2 / 18.2;
+//              128 x 8,000, 42 stages 41.1 / 26.0; 1,000 x 3,000, BF16 65.6 / 25
+//   9,728      784 x 1,024, BF16, 78 stages 29.3 / 24.4; 128 x 8,000, BF16 47.6 / 62.9
+// (With 24 stages as the line, whatever the rows, calls took up to 1.48 times as
+// long as with the fused kernel alone before.)
 bool tc_split_hamming(const TcArgs &a)
 {
-    const int64_t m_tiles = (a.N + tc::BM - 1) / tc::BM;
-    const int kb = (a.ldx * (a.enc == HDC_ENC_BF16 ? 2 : 1) + tc::BKB - 1) / tc::BKB;
-    return a.nb == 1 && a.cls_sign && a.C > 32 && a.C <= tc::H_CMAX && m_tiles * 2 <= sm_count() &&
-           (a.Dk + tc::HBN - 1) / tc::HBN * kb >= 24 && hamming_packed_ok(a.C, a.W);
+    const int64_t m_tiles = (a.N + tc::BM - 1) / tc::BM, sms = sm_count();
+    const int kb = (a.ldx * (a.enc == HDC_ENC_BF16 ? 2 : 1) + tc::BKB - 1) / tc::BKB, nt = (a.Dk + tc::HBN - 1) / tc::HBN;
+    return a.nb == 1 && a.cls_sign && a.C > 32 && a.C <= tc::H_CMAX && m_tiles * 2 <= sms &&
+           (int64_t)nt * kb * (sms - m_tiles) + nt * (sms - 2 * m_tiles) >= 46 * sms && hamming_packed_ok(a.C, a.W);
 }
 
 int64_t tc_split_words(const TcArgs &a) { return tc_split(a) > 1 ? a.N * a.C + (a.N + tc::BM - 1) / tc::BM : 0; }
