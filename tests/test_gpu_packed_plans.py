@@ -29,3 +29,10 @@ def test_distances(N, D, C):
         labels, dd = hdc.hamming_argmin(q, c, D, dists=True, use_ws=use_ws)
         assert torch.equal(dd, ref) and torch.equal(labels.long(), ref.argmin(1))
         assert torch.equal(hdc.hamming_argmin(q, c, D, use_ws=use_ws), labels)
+
+
+# distances of few rows and of class groups of one or two leave as single words
+@pytest.mark.parametrize("N", [1, 31, 33, 64, 65])
+@pytest.mark.parametrize("C", [33, 34, 35, 65, 67, 161, 255])
+def test_distances_of_few_rows(N, C):
+    test_distances(N, 1000, C)
