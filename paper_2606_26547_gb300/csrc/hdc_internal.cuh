@@ -286,7 +286,9 @@ cudaError_t tc_aux_read_status(cudaStream_t st, int *status);
 // turn.  The pointers to what earlier kernels write pass through it: reads
 // through a const pointer are not ordered by the wait alone.  Nor are __ldg
 // and other non-coherent loads, for data that does not change while the kernel
-// runs: these kernels run while the one before them still writes.
+// runs: these kernels run while the one before them still writes.  __ldcg is
+// ordinary in this sense, and what was just written is in L2 (bundling of 100,000 x
+// 16,384 x 100: 76 us with plain loads, 69 with __ldcg).
 template <typename P>
 __device__ __forceinline__ int read_after(P &p)
 {

@@ -276,7 +276,7 @@ __global__ void __launch_bounds__(TW) count_kernel(const uint32_t *__restrict__ 
         const int r0 = off[g] + (it - first[g]) * CH;
         const int n = min(off[g + 1], r0 + CH) - r0;
         __syncthreads();   // the previous item's last stage has been counted
-        for (int r = threadIdx.x; r < n; r += TW) s_rows[r] = perm[r0 + r];
+        for (int r = threadIdx.x; r < n; r += TW) s_rows[r] = __ldcg(perm + r0 + r);
         __syncthreads();
         const int nst = (n + RS - 1) / RS;
         // stage st: rows st*RS .. st*RS + 15 of the item (zero past n and past W)
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(32 * RED_SLICES) reduce_kernel(const uint32_t 
             for (int it = i0 + slice; it < i1; it += RED_SLICES) {
                 const int r0 = o0 + (it - i0) * CH;
                 const int n = min(o1, r0 + CH) - r0;
-                const uint32_t ln = partial[((int64_t)it * W + w) * 8 + j];
+                const uint32_t ln = __ldcg(partial + ((int64_t)it * W + w) * 8 + j);
 #pragma unroll
                 for (int k = 0; k < 4; k++) {
                     const int v = n - 2 * (int)((ln >> (8 * k)) & 0xffu);
