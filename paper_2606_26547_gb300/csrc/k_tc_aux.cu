@@ -123,10 +123,12 @@ cudaError_t launch_packed_rows(tc::HPParams &p, const CUtensorMap &mq, const CUt
 {
     const int sms = hp_sms(), chunks = (p.nt + tc::HP_CHUNK - 1) / tc::HP_CHUNK;
     auto plan = [&](int mt) {
-        return FIN == tc::HP_HAMMING ? hp_plan_hamming(p.N, mt, p.R, p.nt, PRE, sms) : hp_plan_scores(p.N, mt, chunks, sms);
+        return FIN == tc::HP_HAMMING || FIN == tc::HP_FEW ? hp_plan_hamming(p.N, mt, p.R, p.nt, PRE, sms)
+                                                          : hp_plan_scores(p.N, mt, chunks, sms);
     };
     HpPlan pl = plan(1);
-    if (p.R <= 128) {
+    constexpr int MT = FIN == tc::HP_FEW ? 1 : 2;   // few rows are one tile
+    if (MT == 2 && p.R <= 128) {
         const HpPlan p2 = plan(2);
         if (p2.cost < pl.cost) pl = p2;
     }
@@ -139,7 +141,7 @@ cudaError_t launch_packed_rows(tc::HPParams &p, const CUtensorMap &mq, const CUt
     p.nbs = (int)nbs;
     size_t smem = fixed + (PRE ? nbs * atom : tc::hp_nab(pl.mt, false) * atom + (size_t)((p.W + 3) & ~3) * 4);
     if (smem < 120 * 1024) smem = 120 * 1024;
-    auto k = pl.mt == 2 ? tc::tc_hamming_packed_kernel<2, PRE, FIN> : tc::tc_hamming_packed_kernel<1, PRE, FIN>;
+    auto k = pl.mt == 2 ? tc::tc_hamming_packed_kernel<MT, PRE, FIN> : tc::tc_hamming_packed_kernel<1, PRE, FIN>;
     cudaError_t e = allow_smem(k, kMaxSmem);
     if (e != cudaSuccess) return e;
     const int64_t ctas = pl.units * pl.S;
@@ -223,6 +225,8 @@ cudaError_t launch_hamming_packed(const uint32_t *Q, int64_t N, const uint32_t *
     p.kept = end > s0 ? (int)((end - s0 + stride - 1) / stride) : 0;
     p.labels = labels;
     p.dists = dists;
+    if (dists && C % 4 != 0 && N <= 64)
+        return signs ? launch_packed<true, tc::HP_FEW>(p, Q, &mc, st) : launch_packed<false, tc::HP_FEW>(p, Q, nullptr, st);
     return signs ? launch_packed<true, tc::HP_HAMMING>(p, Q, &mc, st) : launch_packed<false, tc::HP_HAMMING>(p, Q, nullptr, st);
 }
 

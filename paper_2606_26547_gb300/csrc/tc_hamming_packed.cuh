@@ -5,7 +5,9 @@
 //   HP_COSINE   the cosine arg-max against b-bit class hypervectors (Sec. 4.2
 //               Algorithmic Choice);
 //   HP_SWEEP    the arg-max of every (class width, perforation) configuration
-//               of a trained model, its correct predictions counted.
+//               of a trained model, its correct predictions counted;
+//   HP_FEW      HP_HAMMING with distances of few rows of a class number that is
+//               no multiple of four, which are not worth staging.
 // A b-bit class value is P signed base-16 digits (1 for up to 4 bits, 2 for 8,
 // 8 for 32), each a class row of its own that E4M3 holds exactly; the digits'
 // dot products, exact in FP32 (at most 8 * 131,072), are put together as
@@ -39,8 +41,9 @@
 //   warp 25     PRE: TMA producer of the class bytes (atoms of R rows x 128
 //               dims) into a ring of p.nbs slots;
 //   warp 26     MMA issuer.
-// PRE: the class rows come already expanded (Cp rows of ldcs bytes, from
-// launch_class_bytes into the caller's workspace).  Without it the expanding
+// PRE: the class rows come already expanded (R rows of bytes in this dim order:
+// class_bytes_kernel's in the caller's workspace, a model's digit rows, or the
+// sweep's).  Without it the expanding
 // warps also expand the class words of every tile into two shared-memory
 // buffers.
 //
@@ -51,9 +54,12 @@
 //
 // TMEM (512 columns): D2 in columns 0..255 (MT x RS columns a buffer, RS = R
 // rounded up to 32), the NAB query buffers of MT x 32 columns from 256.
-// Every wait is bounded as in the encoder.
+// Every barrier wait is bounded as in the encoder.  The cluster barriers of a split
+// row are not: every thread of every rank reaches both, an aborted one too, and
+// the ranks of a cluster run together.
 //
-// What bounds it, and the form before: see launch_hamming_packed.
+// Bound by an atom's barrier, store and MMA-issue latencies one after the other
+// (~420 cycles for 128 dims; no pipe is full).  The forms' times: launch_hamming_packed.
 #pragma once
 #include "tc_hamming.cuh"
 
@@ -70,7 +76,7 @@ constexpr int HP_QB = 3;                       // query chunks in the ring
 constexpr int HP_CHUNK = 4;                    // 256-dim tiles per query chunk (128 bytes of a row)
 constexpr int HP_NBS_MAX = 16;                 // most class-atom slots
 constexpr int HP_SMAX = 8;                     // most CTAs a unit's dims are split over
-constexpr int HP_HAMMING = 0, HP_COSINE = 1, HP_SWEEP = 2;
+constexpr int HP_HAMMING = 0, HP_COSINE = 1, HP_SWEEP = 2, HP_FEW = 3;
 constexpr int HP_MAXCFG = HDC_SWEEP_MAX_STRIDES * HDC_SWEEP_MAX_BITS;
 constexpr uint32_t HP_ACOL = 256;              // first TMEM column of the query buffers
 constexpr int HP_NAB_MAX = 8;                  // query-atom buffers: 4, or 8 with MT = 1 and PRE
@@ -237,6 +243,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     constexpr int QCH = UROWS * 128;                             // bytes of a query chunk
     uint8_t *sQ = smem;
     constexpr int NAB = hp_nab(MT, PRE);
+    constexpr bool HAM = FIN == HP_HAMMING || FIN == HP_FEW;
     uint8_t *sB = smem + hp_q_bytes(MT);                         // class atoms: nbs, or one per query buffer
     const int atom_bytes = p.R * 128;
     int32_t *s_out = reinterpret_cast<int32_t *>(sB + (size_t)(PRE ? p.nbs : NAB) * atom_bytes);   // 4 * MT x HP_OUT
@@ -292,7 +299,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
     // distances are staged there)
     double *s_norm = reinterpret_cast<double *>(s_out), *s_rinv = s_norm + HP_CMAX;
     float *s_rinvf = reinterpret_cast<float *>(s_rinv + HP_CMAX);   // (narrowing takes the FP64 pipe: once here)
-    if (FIN != HP_HAMMING)
+    if (!HAM)
         for (int i = tid; i < (FIN == HP_SWEEP ? p.ncfg : 1) * p.C; i += HP_THREADS) {
             const int f = FIN == HP_SWEEP ? i / p.C : 0;
             const double n = FIN == HP_COSINE ? p.cnorm[i] : sqrt((double)p.sumsq[(int64_t)p.cfg_k[f] * p.C + i % p.C]);
@@ -340,7 +347,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                     for (int i = 0; i < 32; i += 4)
                         if (i < nc && lane < nrow)
                             *reinterpret_cast<uint4 *>(o + i) = make_uint4(v[i], v[i + 1], v[i + 2], v[i + 3]);
-                } else if (p.N <= 64 || nc <= 2) {   // single words: a row of 255 classes 10 us (16 staged)
+                } else if (FIN == HP_FEW) {   // single words: one row of 255 classes 10 us (16 staged)
                     int32_t *o = p.dists + (row0 + lane) * p.C + j * 32;
 #pragma unroll
                     for (int i = 0; i < 32; i++)
@@ -351,6 +358,11 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                     for (int i = 0; i < 32; i++)
                         if (i < nc) out[lane * 33 + i] = (int32_t)v[i];
                     __syncwarp();
+                    if (nc <= 2) {   // a lane its own row (10^6 x 128 dims x 33: 112 us by columns, 91 so)
+                        int32_t *o = p.dists + (row0 + lane) * p.C + j * 32;
+                        for (int i = 0; lane < nrow && i < nc; i++) o[i] = out[lane * 33 + i];
+                        continue;
+                    }
                     int32_t *o = p.dists + row0 * p.C + j * 32 + lane;
                     if (lane < nc)
 #pragma unroll 8
@@ -562,8 +574,8 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             const bool ok = part < 2 && c < p.C && t * 4 < p.W;
             const uint32_t *w = p.cls + (int64_t)(ok ? c : 0) * p.W + (ok ? t * 4 : 0);
             if (!ok) return make_uint4(0, 0, 0, 0);
-            if (MT == 1) return *reinterpret_cast<const uint4 *>(w);
-            const uint2 h = *reinterpret_cast<const uint2 *>(w + part * 2);
+            if (MT == 1) return __ldcg(reinterpret_cast<const uint4 *>(w));
+            const uint2 h = __ldcg(reinterpret_cast<const uint2 *>(w + part * 2));
             return make_uint4(h.x, h.y, 0, 0);
         };
         const int tu0 = ch0 * 2 * HP_CHUNK, tun = min(ch1 * 2 * HP_CHUNK, 2 * p.nt) - tu0;   // a unit's atoms
@@ -638,7 +650,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
             if (!__all_sync(0xffffffffu, okd)) break;
             tc_fence_after();
             const uint32_t dcol = tmem + tlane + (uint32_t)((d2 * MT + (e >> 2)) * RS);
-            if (S == 1 && FIN != HP_HAMMING) {
+            if (S == 1 && !HAM) {
                 finish_scores(u * UROWS + e * 32,
                               [&](int col, uint32_t(&v)[8]) { hp_tmem_ld8(dcol + (uint32_t)col, v); });
             } else if (S == 1) {
@@ -685,7 +697,7 @@ __global__ void __launch_bounds__(HP_THREADS, 1)
                 for (int i = 0; i < decltype(count)::value; i++)
                     v[i] = col + i < p.R ? __float_as_uint(own[(col + i) * UROWS]) : 0u;
             };
-            if (FIN == HP_HAMMING)
+            if (HAM)
                 finish(u0 * UROWS + e * 32, s_out + e * (HP_OUT / 4),
                        [&](int j, uint32_t(&v)[32]) { sums(j * 32, v, HpInt<32>()); });
             else
