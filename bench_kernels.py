@@ -5,8 +5,9 @@ each beside the roofline that bounds it (the numbers under profiles/).
 Subcommands (one JSON line each):
 
   hamming   hdc_hamming_argmin on packed binary hypervectors at the shapes of
-            the retraining and clustering passes.  Up to 16 classes (and above
-            256) the distances are popcounts, bound by the popcount unit (16
+            the retraining and clustering passes.  Up to 16 classes (32 in small
+            calls of narrow rows, and above 256) the distances are popcounts,
+            bound by the popcount unit (16
             results per clock per SM); 17..256 classes run as a tensor-core
             product of the rows expanded to +-1.
   training  hdc_train_epoch: one bundling pass and one retraining epoch
@@ -111,7 +112,7 @@ def hamming(N: int, D: int, C: int, reps: int = 10, seed: int = 0) -> dict:
     Q, Cl = random_rows(N, D, W, g, dev), random_rows(C, D, W, g, dev)
     ms, clk = timed_ms(lambda: hdc.hamming_argmin(Q, Cl, D), reps)
     assert hdc.stream_status() == 0
-    tc = 16 < C <= 256 and W <= 4096
+    tc = 16 < C <= 256 and W <= 4096 and not (C <= 32 and W <= 64 and N * W <= 260000)
     out = {"N": N, "D": D, "C": C, "W": W, "ms": round(ms, 4), "queries_per_s": N / (ms / 1e3),
            "word_compares_per_s": N * C * W / (ms / 1e3),
            "route": "tensor cores (rows expanded to +-1)" if tc else "popcount", "clocks": clk}

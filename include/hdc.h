@@ -204,7 +204,7 @@ hdc_status hdc_hamming_argmin(const uint32_t *Q, const uint32_t *Cls,
  * D <= 131072 (on the tensor-core route), the class hypervectors expanded to
  * one E4M3 +-1 byte per dim (C rounded up to 16 rows of
  * 256 * ceil(W(D) / 8) bytes); 0 for every other C and D (17..32 classes
- * take that route without one).
+ * take that route without one, but for small calls of narrow rows).
  * HDC_ERR_INVALID_ARG for C <= 0, D <= 0 or a NULL bytes.                  */
 hdc_status hdc_hamming_argmin_workspace_bytes(int32_t C, int32_t D, size_t *bytes);
 
@@ -275,8 +275,10 @@ hdc_status hdc_train_apply(const int32_t *delta, int32_t C, int32_t D,
  * labels[i] for X (N x F FP32).  class_bits 1: Hamming arg-min over K,
  * dists (N x C int32, optional).  class_bits > 1: cosine arg-max with
  * score = dot(1-2*q, chat) / ||chat|| over K (IEEE FP64, 0 if the norm is
- * 0), scores (N x C double, optional).  Encoded hypervectors are kept on
- * chip on the tensor-core path and never written to memory.              */
+ * 0), scores (N x C double, optional).  Up to 128 binary classes (and up to
+ * 128 with float queries) on the tensor cores, encoded hypervectors are kept on
+ * chip and never written to memory; small batches of 33..112 binary classes,
+ * b-bit classes of binary queries and more classes are encoded into ws first. */
 hdc_status hdc_classify(const float *X, int64_t N, const hdc_model *m,
                         int32_t *labels, int32_t *dists, double *scores,
                         void *ws, size_t ws_bytes, hdc_stream_t stream);

@@ -46,7 +46,7 @@ constexpr int STEP_ROWS = 64;      // points of a block
 constexpr int STEP_PLANES = 7;     // counts up to STEP_ROWS
 constexpr int STEP_MAXK = 64;
 constexpr int UPD_SLICES = 16;     // most warps of an update block, each a part of the runs
-constexpr int CHIP_SMS = 152;
+constexpr int CHIP_SMS = 152;       // a GB300; not asked for, so that size query and call always agree
 constexpr size_t STEP_SMEM = 200 * 1024;   // most shared memory of an assignment block
 
 // Lines of the route, from both sides timed (us an iteration, 2 / 7 launches): a

@@ -341,7 +341,7 @@ __global__ void __launch_bounds__(LWARPS * 32) levelid_few_kernel(const float *_
 // varying dim) 40 logic operations and 10 POPC at 20 words, where the rows above
 // take 4.7 F / 32 = 91 operations for every dim.
 // 262,144 x 617 x 1,024: 128 levels 2,062 -> 1,080 us, 16 levels 1,998 -> 831;
-// 60,000 x 617 x 10,000, 128 levels 4,707 -> 2,514.  Bound by the logic pipe (72 %
+// 60,000 x 617 x 10,000, 128 levels 4,707 -> 2,514.  Bound by the logic pipe (69 %
 // of its slots; two warps a scheduler, 240 registers a thread).
 
 constexpr int CT = 256;                 // threads of a block
@@ -663,7 +663,7 @@ LevelLayout level_layout(int F, int L, int Wk)
     return Ly;
 }
 
-constexpr int SMS = 152;
+constexpr int SMS = 152;   // a GB300: the lines below were measured on it, and no result depends on it
 constexpr size_t FEW_SMEM = 220 * 1024, ENCODE_SMEM = 200 * 1024;   // most shared memory of a block; of staged rows
 
 template <int NFW>

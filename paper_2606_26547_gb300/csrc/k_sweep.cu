@@ -276,8 +276,6 @@ struct SweepRows {
     int jb[MAXB * MAXS], entry[MAXB * MAXS], digits[MAXB * MAXS], row[MAXB * MAXS];
 };
 
-__device__ __forceinline__ uint32_t entry_mask(const SweepConf &cf, int i, int w);
-
 // A block takes one class, 1,024 dims (a thread four dims of one word) and one
 // width, after scanning all of the class's accumulators for its largest
 // magnitude; the squares of the kept values are added into sumsq (zeroed by the
